@@ -324,8 +324,7 @@ struct Factorizer {
       float* dx = (float*)scratch().alloc(feat.size() / 2 + 1);
       float* dy = (float*)scratch().alloc(evs.size() / 2 + 1);
       CK(cudaMemcpyAsync(dx, feat.data(), sizeof(float) * feat.size(), cudaMemcpyHostToDevice, s));
-      float* dwk = (float*)scratch().alloc(mlp_predict_floats((int)evs.size()) / 2 + 1);
-      mlp_predict_device(d_mlp, dx, dy, (int)evs.size(), s, dwk);
+      mlp_predict_device(d_mlp, dx, dy, (int)evs.size(), s);
       float* hpred = (float*)st.host_alloc(sizeof(float) * evs.size());
       CK(cudaMemcpyAsync(hpred, dy, sizeof(float) * evs.size(), cudaMemcpyDeviceToHost, s));
       wait();
