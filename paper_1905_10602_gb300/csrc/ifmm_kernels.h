@@ -37,7 +37,10 @@ void launch_bd_fill(DescStage& st, const std::vector<BdBlockDesc>& v, const doub
 void launch_interp(DescStage& st, const std::vector<InterpDesc>& v, const double* pts, int N, int p, int dof);
 void launch_m2l_table(cudaStream_t s, double* out, int p, double h, const ifmm_kernel& k);
 void launch_m2m_table(cudaStream_t s, double* out, int p, int dof);
-void launch_matvec(cudaStream_t s, const double* pts, int N, const double* x, double* y, const ifmm_kernel& k);
+// part: matvec_part_doubles(N, k) doubles of partial sums, or NULL where that is 0
+size_t matvec_part_doubles(int n, const ifmm_kernel& k);
+void launch_matvec(cudaStream_t s, const double* pts, int N, const double* x, double* y, const ifmm_kernel& k,
+                   double* part);
 void launch_split_df(cudaStream_t s, const double* in, float* hi, float* lo, int n);
 // part: the symmetric kernel's partial sums (matvec_sym_part_floats(N) floats,
 // as float2), or NULL where none was allocated (the symmetric candidate is then

@@ -8,6 +8,7 @@
 
 #include "dense.cuh"
 #include "pairs.cuh"
+#include "matvec_fp64.cuh"
 #include "ifmm_kernels.h"
 #include "runtime.h"
 
@@ -2091,14 +2092,33 @@ void launch_m2m_table(cudaStream_t s, double* out, int p, int dof) {
   check_launch("k_m2m_table");
 }
 
-void launch_matvec(cudaStream_t s, const double* pts, int N, const double* x, double* y, const ifmm_kernel& k) {
+size_t matvec_part_doubles(int n, const ifmm_kernel& k) { return matvec64_part_doubles(n, kernel_dof(k)); }
+
+void launch_matvec(cudaStream_t s, const double* pts, int N, const double* x, double* y, const ifmm_kernel& k,
+                   double* part) {
   cudaEvent_t pe = profiler().begin(KK_MATVEC, s);
-  if (kernel_dof(k) == 2)
+  const double *px = pts, *py = pts + N, *pz = pts + 2 * (long)N;
+  const int dof = kernel_dof(k);
+  if (part) {
+    const int tb = matvec64_tile(N);
+    const long T = ((long)N + tb - 1) / tb;
+    const unsigned g = (unsigned)(T * (T + 1) / 2);
+    if (dof == 2 && tb == 64)
+      k_matvec64_sym<64, true><<<g, 64, 0, s>>>(px, py, pz, x, part, N, (int)T, k.wavenumber);
+    else if (dof == 2)
+      k_matvec64_sym<128, true><<<g, 128, 0, s>>>(px, py, pz, x, part, N, (int)T, k.wavenumber);
+    else if (tb == 64)
+      k_matvec64_sym<64, false><<<g, 64, 0, s>>>(px, py, pz, x, part, N, (int)T, 0.0);
+    else
+      k_matvec64_sym<128, false><<<g, 128, 0, s>>>(px, py, pz, x, part, N, (int)T, 0.0);
+    k_matvec64_sum<<<(unsigned)(((long)N * dof + 127) / 128), 128, 0, s>>>(part, N, (int)T, x, y, k.scale, k.diag,
+                                                                           k.diag_im, dof);
+  } else if (dof == 2)
     k_matvec_c<<<(N + 255) / 256, 256, 0, s>>>(pts, pts + N, pts + 2 * (long)N, x, y, N, k.scale, k.diag, k.diag_im,
                                                k.wavenumber);
   else
     k_matvec<<<(N + 255) / 256, 256, 0, s>>>(pts, pts + N, pts + 2 * (long)N, x, y, N, k.scale, k.diag);
-  check_launch("k_matvec");
+  check_launch("k_matvec", part ? 2 : 1);
   profiler().end(KK_MATVEC, s, pe);
 }
 

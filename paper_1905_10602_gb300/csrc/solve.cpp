@@ -546,7 +546,8 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
       const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, q, a, b, N, k, part);
       launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, part);
     } else {
-      launch_matvec(s, t->d_pts, (int)NP, a, b, *k);
+      const size_t np = matvec_part_doubles((int)NP, *k);
+      launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? V.get(np) : nullptr);
     }
     if (dev) {
       launch_scatter_perm(s, b, t->d_perm, y, (int)NP, dof);
@@ -619,6 +620,9 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     // the symmetric matvec's partial sums, unless this tree took another kernel
     float2* sympart = nullptr;
     if (df_mv && (!t->matvec_block || (t->matvec_block >> 16) == 3)) sympart = sym_part(Vm, N);
+    // the FP64 matvec's partial sums
+    const size_t np64 = k->arith == IFMM_ARITH_FP64 ? matvec_part_doubles((int)NP, *k) : 0;
+    double* part64 = np64 ? Vm.get(np64) : nullptr;
     FmmPlan* fmm = k->arith == IFMM_ARITH_FMM
                        ? fmm_plan(*const_cast<ifmm_tree*>(t), k->order ? k->order : 4, k->scale, k->diag, s)
                        : nullptr;
@@ -631,7 +635,7 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
         const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, qdf, in, out, N, k, sympart);
         launch_matvec_df(s, t->d_pts_df, qdf, qdf + N, in, out, (int)N, k->scale, k->diag, tile, sympart);
       } else {
-        launch_matvec(s, t->d_pts, (int)NP, in, out, *k);
+        launch_matvec(s, t->d_pts, (int)NP, in, out, *k, part64);
       }
     };
     CK(cudaMemsetAsync(xt, 0, sizeof(double) * N, s));
