@@ -1,6 +1,6 @@
 // Batched dense linear algebra used by every step of the factorization and
 // the solve: block copies, variable-size GEMM, Gauss-Jordan inversion with
-// partial pivoting, Householder QR (R factor), one-sided Jacobi SVD, GEMV.
+// partial pivoting, Householder QR (R factor), one-sided Jacobi SVD.
 //
 // Every matrix is column-major with a leading dimension (BLAS convention).
 // One descriptor describes one problem; a launch covers a batch of problems of
@@ -2178,45 +2178,6 @@ __global__ void k_frob(const FrobDesc* __restrict__ d, int nd) {
   }
   s = block_sum(s, scratch);
   if (threadIdx.x == 0) D.out[0] = sqrt(s);
-}
-
-// ---------------------------------------------------------------- GEMV
-// 4 independent accumulators over the columns of a column-major block: row i,
-// columns [0, n) of A (leading dimension lda) against x.
-__device__ __forceinline__ double dot_row(const double* __restrict__ a, long lda, const double* __restrict__ x, int n) {
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  int j = 0;
-  for (; j + 3 < n; j += 4) {
-    s0 += a[(long)j * lda] * x[j];
-    s1 += a[(long)(j + 1) * lda] * x[j + 1];
-    s2 += a[(long)(j + 2) * lda] * x[j + 2];
-    s3 += a[(long)(j + 3) * lda] * x[j + 3];
-  }
-  for (; j < n; ++j) s0 += a[(long)j * lda] * x[j];
-  return (s0 + s1) + (s2 + s3);
-}
-
-// y = alpha * op(A) x + beta * y.  Non-transposed: a thread per row walks the
-// columns (consecutive threads read consecutive rows of a column).  Transposed:
-// a warp per output reduces one contiguous column of A.
-__global__ void k_gemv(const GemvDesc* __restrict__ d, int nd) {
-  if ((int)blockIdx.x >= nd) return;
-  const GemvDesc D = d[blockIdx.x];
-  if (D.trans) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    for (int i = w; i < D.n; i += nw) {
-      const double* a = D.A + (long)i * D.lda;
-      double s = 0.0;
-      for (int j = lane; j < D.m; j += 32) s += a[j] * D.x[j];
-      s = warp_sum(s);
-      if (lane == 0) D.y[i] = (D.beta == 0.0) ? D.alpha * s : D.alpha * s + D.beta * D.y[i];
-    }
-  } else {
-    for (int i = threadIdx.x; i < D.m; i += blockDim.x) {
-      const double s = dot_row(D.A + i, D.lda, D.x, D.n);
-      D.y[i] = (D.beta == 0.0) ? D.alpha * s : D.alpha * s + D.beta * D.y[i];
-    }
-  }
 }
 
 }  // namespace ifmm

@@ -41,15 +41,6 @@ struct QrDesc {
   int ld, m, n;
 };
 
-// y = alpha * op(A) x + beta * y ; A is m x n (op(A) is n x m when trans).
-struct GemvDesc {
-  const double* A;
-  const double* x;
-  double* y;
-  int lda, m, n, trans;
-  double alpha, beta;
-};
-
 // One operation of the IFMM solve (Algorithm 2): for r in [0, rows)
 //   out[o(r)] = beta * base[o(r)] + alpha * sum_{c < ncols} M[r * ldm + c] * v(c),
 // v(c) = x[c] (xidx == nullptr) or x[xidx[c]], o(r) = r (oidx == nullptr) or

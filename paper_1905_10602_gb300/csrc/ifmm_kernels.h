@@ -84,6 +84,22 @@ void launch_fmm_l2l(cudaStream_t s, const int* parent, const int* cells, const d
 void launch_fmm_l2p(cudaStream_t s, const double* S, const long* soff, const int* leaf_ptr, const int* nbr_ptr,
                     const int* nbr, const double* L, const double* pts, int N, const double* x, double* y, int nleaf,
                     int rc, double scale, double diag);
+// GMRES vector operations (krylov.cuh).  part: kry_parts(n) doubles per vector
+// named below; norm2, h: device results.
+int kry_parts(long n);
+// norm2 = w . w and v = w / |w| (untouched when |w| is not positive); part: 1 vector
+void launch_kry_norm(cudaStream_t s, const double* w, long n, double* part, double* norm2, double* v);
+// one Arnoldi step, classical Gram-Schmidt twice against the nv vectors V: h[0..nv)
+// and h[nv..2 nv) the two passes' coefficients, h[2 nv] = |w|^2 after them, vnext =
+// w / |w|; part: 2 nv vectors
+void launch_kry_arnoldi(cudaStream_t s, const double* V, long n, int nv, double* w, double* part, double* h,
+                        double* vnext);
+// u = V y
+void launch_kry_combine(cudaStream_t s, const double* V, long n, int nv, const double* y, double* u);
+// x += z
+void launch_kry_add(cudaStream_t s, const double* z, double* x, long n);
+// r = b - r, norm2 = r . r, v = r / |r|; part: 1 vector
+void launch_kry_residual(cudaStream_t s, const double* b, double* r, long n, double* part, double* norm2, double* v);
 const char* last_error();
 
 }  // namespace ifmm

@@ -9,6 +9,7 @@
 #include "dense.cuh"
 #include "pairs.cuh"
 #include "matvec_fp64.cuh"
+#include "krylov.cuh"
 #include "ifmm_kernels.h"
 #include "runtime.h"
 
@@ -994,20 +995,57 @@ void launch_frob(DescStage& st, const std::vector<FrobDesc>& v) {
   check_launch("k_frob");
 }
 
-void launch_gemv(DescStage& st, const std::vector<GemvDesc>& v) {
-  if (v.empty()) return;
-  for (size_t i = 0; i < v.size() && registry().on; ++i) {
-    const GemvDesc& x = v[i];
-    req(x.A, span(x.m, x.n, x.lda), "gemv.A", i);
-    req(x.x, sizeof(double) * (x.trans ? x.m : x.n), "gemv.x", i);
-    req(x.y, sizeof(double) * (x.trans ? x.n : x.m), "gemv.y", i);
-  }
-  const GemvDesc* d = st.push(v);
-  prof_batch_tag() = (long)v.size();
-  cudaEvent_t pe = profiler().begin(KK_GEMV, st.stream);
-  k_gemv<<<(unsigned)v.size(), 128, 0, st.stream>>>(d, (int)v.size());
-  check_launch("k_gemv");
-  profiler().end(KK_GEMV, st.stream, pe);
+// ------------------------------------------------------------------ GMRES vectors
+// Chunk of a vector per CTA: two CTAs per SM, at least 512 elements (below that
+// a CTA is all latency), at most what its shared memory holds.
+int kry_chunk(long n) {
+  const long c = ((n + 303) / 304 + 255) / 256 * 256;
+  return (int)std::min<long>(kKryMaxChunk, std::max<long>(512, c));
+}
+int kry_parts(long n) { return (int)((n + kry_chunk(n) - 1) / kry_chunk(n)); }
+
+void launch_kry_norm(cudaStream_t s, const double* w, long n, double* part, double* norm2, double* v) {
+  const int c = kry_chunk(n), nb = kry_parts(n);
+  cudaEvent_t pe = profiler().begin(KK_GEMV, s, 2);
+  k_kry_dots<<<nb, kKryThreads, sizeof(double) * c, s>>>(w, n, 1, w, c, part);
+  k_kry_scale<<<nb, kKryThreads, 0, s>>>(w, n, c, part, norm2, v);
+  check_launch("k_kry", 2);
+  profiler().end(KK_GEMV, s, pe);
+}
+
+void launch_kry_arnoldi(cudaStream_t s, const double* V, long n, int nv, double* w, double* part, double* h,
+                        double* vnext) {
+  const int c = kry_chunk(n), nb = kry_parts(n);
+  double* p2 = part + (long)nv * nb;
+  const size_t sm = sizeof(double) * c, smh = sizeof(double) * (c + nv);
+  cudaEvent_t pe = profiler().begin(KK_GEMV, s, 4);
+  k_kry_dots<<<nb, kKryThreads, sm, s>>>(V, n, nv, w, c, part);
+  k_kry_update<<<nb, kKryThreads, smh, s>>>(V, n, nv, w, c, part, h, p2, 0);
+  k_kry_update<<<nb, kKryThreads, smh, s>>>(V, n, nv, w, c, p2, h + nv, part, 1);
+  k_kry_scale<<<nb, kKryThreads, 0, s>>>(w, n, c, part, h + 2 * nv, vnext);
+  check_launch("k_kry", 4);
+  profiler().end(KK_GEMV, s, pe);
+}
+
+void launch_kry_combine(cudaStream_t s, const double* V, long n, int nv, const double* y, double* u) {
+  cudaEvent_t pe = profiler().begin(KK_GEMV, s);
+  k_kry_combine<<<(unsigned)((n + kKryThreads - 1) / kKryThreads), kKryThreads, 0, s>>>(V, n, nv, y, u);
+  check_launch("k_kry_combine");
+  profiler().end(KK_GEMV, s, pe);
+}
+
+void launch_kry_add(cudaStream_t s, const double* z, double* x, long n) {
+  k_kry_add<<<(unsigned)((n + kKryThreads - 1) / kKryThreads), kKryThreads, 0, s>>>(z, x, n);
+  check_launch("k_kry_add");
+}
+
+void launch_kry_residual(cudaStream_t s, const double* b, double* r, long n, double* part, double* norm2, double* v) {
+  const int c = kry_chunk(n), nb = kry_parts(n);
+  cudaEvent_t pe = profiler().begin(KK_GEMV, s, 2);
+  k_kry_residual<<<nb, kKryThreads, sizeof(double) * c, s>>>(b, r, n, c, part);
+  k_kry_scale<<<nb, kKryThreads, 0, s>>>(r, n, c, part, norm2, v);
+  check_launch("k_kry_residual", 2);
+  profiler().end(KK_GEMV, s, pe);
 }
 
 // ------------------------------------------------------------------ IFMM kernels

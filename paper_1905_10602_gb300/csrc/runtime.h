@@ -62,7 +62,26 @@ Registry& registry();
 bool poison_on();
 void poison_fill(void* p, size_t bytes);
 
-// Bump allocator over cudaMalloc'd chunks.  reset() makes the memory reusable;
+// Memory that outlives one call: device blocks from a library-owned CUDA memory
+// pool per device and pinned host chunks, kept for the next call instead of
+// going back to the driver each time (an allocation and its release cost 0.2 ms
+// for a workspace, 0.3 ms for a 256 MB chunk, 3.2 ms for 64 MB of pinned memory;
+// a job takes a few dozen).  Bounded: at most 16 GiB of unused device memory (of 280) and
+// 256 MiB of unused pinned memory stay, and all of it is given back when the
+// process' last tree is freed, or when an allocation fails for want of memory.
+// Safe from any thread and stream: a block is handed out free of pending work,
+// and pool_free / pinned_free are only called once the work that used the block
+// has finished (see pool_quiesce).
+void* pool_alloc(size_t bytes);            // current device; throws IFMM_ENOMEM
+void pool_free(void* p);
+void* pinned_alloc(size_t bytes, size_t* got);  // at least bytes; *got = the chunk's size
+void pinned_free(void* p, size_t got);
+void pool_tree_count(int delta);           // live trees of the process
+// For releases while an exception passes: work that was issued may still use
+// the memory, so the device is waited for first.
+void pool_quiesce();
+
+// Bump allocator over chunks of the pool.  reset() makes the memory reusable;
 // callers only reset at points where all earlier work on the stream that uses
 // the memory has been ordered before later work (one stream) .
 struct DeviceArena {
@@ -90,7 +109,7 @@ struct DeviceArena {
     }
     size_t sz = std::max(min_chunk, bytes);
     void* p = nullptr;
-    CK(cudaMalloc(&p, sz));
+    p = pool_alloc(sz);
     chunks.push_back({(char*)p, sz});
     ci = chunks.size() - 1;
     off = bytes;
@@ -106,8 +125,9 @@ struct DeviceArena {
     off = 0;
   }
   void release() {
+    if (!chunks.empty()) pool_quiesce();
     for (auto& c : chunks) registry().remove_range(c.p, c.size);
-    for (auto& c : chunks) cudaFree(c.p);
+    for (auto& c : chunks) pool_free(c.p);
     chunks.clear();
     ci = off = 0;
   }
@@ -144,9 +164,9 @@ struct DescStage {
       ++hci;
       hoff = 0;
     }
-    size_t sz = std::max<size_t>((size_t)64 << 20, bytes);
-    void* p = nullptr;
-    CK(cudaMallocHost(&p, sz));
+    size_t sz = 0;
+    // the first chunk small (a launch or a small job needs no more), then larger
+    void* p = pinned_alloc(std::max(bytes, (size_t)(host.empty() ? 4 : 32) << 20), &sz);
     host.push_back({(char*)p, sz});
     hci = host.size() - 1;
     hoff = bytes;
@@ -177,7 +197,8 @@ struct DescStage {
     dev.reset();
   }
   void release() {
-    for (auto& h : host) cudaFreeHost(h.first);
+    if (!host.empty()) pool_quiesce();
+    for (auto& h : host) pinned_free(h.first, h.second);
     host.clear();
     dev.release();
   }
@@ -227,7 +248,6 @@ void launch_copy_sorted(DescStage& st, const CopyDesc* h, size_t ns, size_t nb);
 void launch_gemm(DescStage& st, const std::vector<GemmDesc>& v, int prec);
 void launch_inv(DescStage& st, const std::vector<InvDesc>& v);
 void launch_qr(DescStage& st, const std::vector<QrDesc>& v, int prec);
-void launch_gemv(DescStage& st, const std::vector<GemvDesc>& v);
 void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec);
 void launch_svd_rt(DescStage& st, const std::vector<SvdRtDesc>& v, int prec);
 void launch_sketch(DescStage& st, const std::vector<SketchDesc>& v);
@@ -265,21 +285,6 @@ inline GemmDesc gmm(const double* A, int lda, int ta, const double* B, int ldb, 
   d.k = k;
   d.ta = ta;
   d.tb = tb;
-  d.alpha = alpha;
-  d.beta = beta;
-  return d;
-}
-
-inline GemvDesc gmv(const double* A, int lda, int m, int n, int trans, const double* x, double* y, double alpha,
-                    double beta) {
-  GemvDesc d;
-  d.A = A;
-  d.lda = lda;
-  d.m = m;
-  d.n = n;
-  d.trans = trans;
-  d.x = x;
-  d.y = y;
   d.alpha = alpha;
   d.beta = beta;
   return d;

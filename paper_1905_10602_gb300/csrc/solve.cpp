@@ -390,6 +390,7 @@ void ifmm_tree::ensure_device() {
   for (int64_t i = 0; i < N; ++i)
     for (int d = 0; d < 3; ++d) soa[(size_t)d * N + i] = pts[3 * i + d];
   CK(cudaMalloc(&d_pts, sizeof(double) * 3 * N));
+  pool_tree_count(1);
   CK(cudaMemcpy(d_pts, soa.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice));
   CK(cudaMalloc(&d_perm, sizeof(int32_t) * N));
   CK(cudaMemcpy(d_perm, perm.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
@@ -414,6 +415,7 @@ ifmm_tree::~ifmm_tree() {
   if (d_pts) {
     registry().remove_range(d_pts, sizeof(double) * 3 * N);
     cudaFree(d_pts);
+    pool_tree_count(-1);
   }
   if (d_perm) {
     registry().remove_range(d_perm, sizeof(int32_t) * N);
@@ -425,51 +427,40 @@ ifmm_tree::~ifmm_tree() {
   }
 }
 
-// device buffers for the GMRES / solve wrappers
+// Device buffers of one call, carved from one block of the pool: reserve() every
+// piece first, then get() them.
 struct Vecs {
-  std::vector<std::pair<double*, size_t>> p;
-  ~Vecs() {
-    for (auto x : p) {
-      registry().remove_range(x.first, x.second);
-      cudaFree(x.first);
-    }
-  }
+  char* base = nullptr;
+  size_t total = 0, off = 0;
+  static size_t up(size_t n) { return (sizeof(double) * std::max<size_t>(n, 1) + 255) & ~(size_t)255; }
+  void reserve(size_t n) { total += up(n); }
   double* get(size_t n) {
-    double* x = nullptr;
-    const size_t bytes = sizeof(double) * std::max<size_t>(n, 1);
-    CK(cudaMalloc(&x, bytes));
-    registry().add(x, bytes);
-    p.push_back({x, bytes});
+    if (!base) base = (char*)pool_alloc(std::max<size_t>(total, 256));
+    IFMM_REQUIRE(off + up(n) <= total, IFMM_EINVAL, "internal: workspace larger than reserved");
+    double* x = (double*)(base + off);
+    off += up(n);
+    registry().add(x, sizeof(double) * std::max<size_t>(n, 1));
     return x;
   }
+  Vecs() = default;
+  Vecs(const Vecs&) = delete;
+  Vecs& operator=(const Vecs&) = delete;
+  ~Vecs() {
+    if (!base) return;
+    pool_quiesce();
+    registry().remove_range(base, total);
+    pool_free(base);
+  }
 };
 
-// partial-sum buffer of the symmetric float-pair matvec, when it is at most
-// 8 GiB (N up to about 300,000 points); NULL otherwise
-static float2* sym_part(Vecs& V, int64_t N) {
-  const size_t floats = matvec_sym_part_floats((int)N);
-  if (floats * sizeof(float) > ((size_t)8 << 30)) return nullptr;
-  return (float2*)V.get(floats / 2);
+// doubles of the partial-sum buffer of the symmetric float-pair matvec, when it
+// is at most 8 GiB (N up to about 300,000 points) and this tree may take that
+// kernel; 0 otherwise
+static size_t sym_part_doubles(const ifmm_tree& t) {
+  if (t.matvec_block && (t.matvec_block >> 16) != 3) return 0;
+  const size_t floats = matvec_sym_part_floats((int)t.N);
+  return floats * sizeof(float) > ((size_t)8 << 30) ? 0 : floats / 2;
 }
-
-// dot products / norms on the device through the GEMV kernel, read on the host
-struct Blas1 {
-  cudaStream_t s;
-  DescStage st;
-  double* d_out;
-  double* h_out;
-  explicit Blas1(cudaStream_t s_) : s(s_) {
-    st.stream = s;
-    CK(cudaMalloc(&d_out, sizeof(double) * 64));
-    registry().add(d_out, sizeof(double) * 64);
-    CK(cudaMallocHost(&h_out, sizeof(double) * 64));
-  }
-  ~Blas1() {
-    registry().remove_range(d_out, sizeof(double) * 64);
-    cudaFree(d_out);
-    cudaFreeHost(h_out);
-  }
-};
 
 extern "C" {
 
@@ -484,6 +475,7 @@ ifmm_status ifmm_solve(const ifmm_fact* f, const double* r, double* v, int nrhs,
     const bool dev = is_device_ptr(r);
     IFMM_REQUIRE(dev == is_device_ptr(v), IFMM_EINVAL, "r and v must both be host or both device");
     Vecs V;
+    for (int i = 0; i < 2; ++i) V.reserve(N);
     double* a = V.get(N);
     double* b = V.get(N);
     for (int c = 0; c < nrhs; ++c) {
@@ -525,7 +517,12 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
     const int64_t NP = t->N, N = NP * dof;
     const bool dev = is_device_ptr(x);
     IFMM_REQUIRE(dev == is_device_ptr(y), IFMM_EINVAL, "x and y must both be host or both device");
+    const bool df_mv = k->arith == IFMM_ARITH_DF, fmm_mv = k->arith == IFMM_ARITH_FMM;
+    // partial sums of the symmetric kernels
+    const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
     Vecs V;
+    for (int i = 0; i < (df_mv ? 4 : 3); ++i) V.reserve(N);
+    if (np) V.reserve(np);
     double* a = V.get(N);
     double* b = V.get(N);
     double* c = V.get(N);
@@ -535,18 +532,17 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
       src = c;
     }
     launch_gather_perm(s, src, t->d_perm, a, (int)NP, dof);
-    if (k->arith == IFMM_ARITH_FMM) {
+    if (fmm_mv) {
       FmmPlan* P = fmm_plan(*const_cast<ifmm_tree*>(t), k->order ? k->order : 4, k->scale, k->diag, s);
       fmm_apply(*t, *P, a, b, s);
-    } else if (k->arith == IFMM_ARITH_DF) {
+    } else if (df_mv) {
       float* q = (float*)V.get(N);
       launch_split_df(s, a, q, q + N, (int)N);
       ifmm_tree* tm = const_cast<ifmm_tree*>(t);
-      float2* part = (!tm->matvec_block || (tm->matvec_block >> 16) == 3) ? sym_part(V, N) : nullptr;
+      float2* part = np ? (float2*)V.get(np) : nullptr;
       const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, q, a, b, N, k, part);
       launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, part);
     } else {
-      const size_t np = matvec_part_doubles((int)NP, *k);
       launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? V.get(np) : nullptr);
     }
     if (dev) {
@@ -583,98 +579,88 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     const int m = restart;
     const bool dev = is_device_ptr(b);
     IFMM_REQUIRE(dev == is_device_ptr(x), IFMM_EINVAL, "b and x must both be host or both device");
+    const bool df_mv = k->arith == IFMM_ARITH_DF, fmm_mv = k->arith == IFMM_ARITH_FMM;
+    // the symmetric matvec's partial sums (float pairs, unless this tree took
+    // another kernel, or FP64)
+    const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
+    const size_t nkp = (size_t)kry_parts(N) * 2 * m;
     Vecs Vm;
+    for (int i = 0; i < 6; ++i) Vm.reserve(N);
+    Vm.reserve((size_t)N * (m + 1));
+    Vm.reserve(2 * (size_t)m + 2);
+    Vm.reserve(nkp);
+    if (df_mv) Vm.reserve(N);
+    if (np) Vm.reserve(np);
     double* bt = Vm.get(N);   // b in tree order
     double* xt = Vm.get(N);   // x in tree order
     double* rt = Vm.get(N);
     double* wt = Vm.get(N);
     double* zt = Vm.get(N);
     double* Vb = Vm.get((size_t)N * (m + 1));
-    double* hv = Vm.get((size_t)2 * (m + 2));
+    double* hv = Vm.get((size_t)2 * m + 2);
+    double* kp = Vm.get(nkp);
     double* tmp = Vm.get(N);
-    Blas1 B(s);
+    float* qdf = df_mv ? (float*)Vm.get(N) : nullptr;
+    double* part = np ? Vm.get(np) : nullptr;
     const double* src = b;
     if (!dev) {
       CK(cudaMemcpyAsync(tmp, b, sizeof(double) * N, cudaMemcpyHostToDevice, s));
       src = tmp;
     }
     launch_gather_perm(s, src, t->d_perm, bt, (int)NP, dof);
-    auto dot = [&](const double* u, const double* v) -> double {
-      std::vector<GemvDesc> g{gmv(u, (int)N, (int)N, 1, 1, v, B.d_out, 1.0, 0.0)};
-      launch_gemv(B.st, g);
-      CK(cudaMemcpyAsync(B.h_out, B.d_out, sizeof(double), cudaMemcpyDeviceToHost, s));
+    std::vector<double> hh(2 * (size_t)m + 2);
+    // reads n results back
+    auto fetch = [&](size_t n) {
+      CK(cudaMemcpyAsync(hh.data(), hv, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
-      B.st.reset();
-      return B.h_out[0];
-    };
-    auto axpby = [&](double alpha, const double* u, double beta, double* v) {
-      std::vector<CopyDesc> c{cpy(u, (int)N, v, (int)N, (int)N, 1, alpha, beta)};
-      launch_copy(B.st, c);
     };
     auto precond = [&](const double* in, double* out) {
       if (pre) run_solve_tree(*pre, in, out, s);
       else CK(cudaMemcpyAsync(out, in, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
     };
-    const bool df_mv = k->arith == IFMM_ARITH_DF;
-    float* qdf = df_mv ? (float*)Vm.get(N) : nullptr;
-    // the symmetric matvec's partial sums, unless this tree took another kernel
-    float2* sympart = nullptr;
-    if (df_mv && (!t->matvec_block || (t->matvec_block >> 16) == 3)) sympart = sym_part(Vm, N);
-    // the FP64 matvec's partial sums
-    const size_t np64 = k->arith == IFMM_ARITH_FP64 ? matvec_part_doubles((int)NP, *k) : 0;
-    double* part64 = np64 ? Vm.get(np64) : nullptr;
-    FmmPlan* fmm = k->arith == IFMM_ARITH_FMM
-                       ? fmm_plan(*const_cast<ifmm_tree*>(t), k->order ? k->order : 4, k->scale, k->diag, s)
-                       : nullptr;
+    FmmPlan* fmm =
+        fmm_mv ? fmm_plan(*const_cast<ifmm_tree*>(t), k->order ? k->order : 4, k->scale, k->diag, s) : nullptr;
     auto Amul = [&](const double* in, double* out) {
       if (fmm) {
         fmm_apply(*t, *fmm, in, out, s);
       } else if (df_mv) {
         launch_split_df(s, in, qdf, qdf + N, (int)N);
         ifmm_tree* tm = const_cast<ifmm_tree*>(t);
-        const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, qdf, in, out, N, k, sympart);
-        launch_matvec_df(s, t->d_pts_df, qdf, qdf + N, in, out, (int)N, k->scale, k->diag, tile, sympart);
+        const int tile =
+            tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, qdf, in, out, N, k, (float2*)part);
+        launch_matvec_df(s, t->d_pts_df, qdf, qdf + N, in, out, (int)N, k->scale, k->diag, tile, (float2*)part);
       } else {
-        launch_matvec(s, t->d_pts, (int)NP, in, out, *k, part64);
+        launch_matvec(s, t->d_pts, (int)NP, in, out, *k, part);
       }
     };
     CK(cudaMemsetAsync(xt, 0, sizeof(double) * N, s));
-    CK(cudaMemcpyAsync(rt, bt, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
-    const double bnorm = std::sqrt(dot(bt, bt));
+    // the residual of x = 0 is b
+    launch_kry_norm(s, bt, N, kp, hv, Vb);
+    fetch(1);
+    const double bnorm = std::sqrt(hh[0]);
     IFMM_REQUIRE(bnorm > 0, IFMM_EINVAL, "b is zero");
     int its = 0;
-    double rel = 1.0;
+    double beta = bnorm, rel = 1.0;
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1);
+    // at the top of the loop Vb holds the residual's direction and beta its norm
     while (its < maxit) {
-      const double beta = std::sqrt(dot(rt, rt));
       rel = beta / bnorm;
       if (rel <= tol) break;
       std::fill(H.begin(), H.end(), 0.0);
       std::fill(g.begin(), g.end(), 0.0);
       g[0] = beta;
-      axpby(1.0 / beta, rt, 0.0, Vb);
       int kdone = 0;
       for (int j = 0; j < m; ++j) {
         double* vj = Vb + (size_t)j * N;
         precond(vj, zt);
         Amul(zt, wt);
         ++its;
-        // classical Gram-Schmidt, twice
-        std::vector<double> h(j + 1, 0.0);
-        for (int pass = 0; pass < 2; ++pass) {
-          std::vector<GemvDesc> gg{gmv(Vb, (int)N, (int)N, j + 1, 1, wt, hv, 1.0, 0.0)};
-          launch_gemv(B.st, gg);
-          CK(cudaMemcpyAsync(B.h_out, hv, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-          std::vector<GemvDesc> g2{gmv(Vb, (int)N, (int)N, j + 1, 0, hv, wt, -1.0, 1.0)};
-          launch_gemv(B.st, g2);
-          CK(cudaStreamSynchronize(s));
-          B.st.reset();
-          for (int i = 0; i <= j; ++i) h[i] += B.h_out[i];
-        }
-        const double hn = std::sqrt(dot(wt, wt));
-        for (int i = 0; i <= j; ++i) H[i + (size_t)j * (m + 1)] = h[i];
+        // classical Gram-Schmidt, twice; the next basis vector
+        launch_kry_arnoldi(s, Vb, N, j + 1, wt, kp, hv, vj + N);
+        fetch(2 * (size_t)(j + 1) + 1);
+        const double hn = std::sqrt(hh[2 * (j + 1)]);
+        for (int i = 0; i <= j; ++i) H[i + (size_t)j * (m + 1)] = hh[i] + hh[j + 1 + i];
         H[j + 1 + (size_t)j * (m + 1)] = hn;
-        if (hn > 0) axpby(1.0 / hn, wt, 0.0, Vb + (size_t)(j + 1) * N);
         for (int i = 0; i < j; ++i) {
           double& a = H[i + (size_t)j * (m + 1)];
           double& c = H[i + 1 + (size_t)j * (m + 1)];
@@ -702,19 +688,15 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
         y[i] = sacc / H[i + (size_t)i * (m + 1)];
       }
       CK(cudaMemcpyAsync(hv, y.data(), sizeof(double) * kdone, cudaMemcpyHostToDevice, s));
-      std::vector<GemvDesc> gu{gmv(Vb, (int)N, (int)N, kdone, 0, hv, wt, 1.0, 0.0)};
-      launch_gemv(B.st, gu);
+      launch_kry_combine(s, Vb, N, kdone, hv, wt);
       precond(wt, zt);
-      axpby(1.0, zt, 1.0, xt);
+      launch_kry_add(s, zt, xt, N);
       Amul(xt, rt);
-      axpby(1.0, bt, -1.0, rt);
-      CK(cudaStreamSynchronize(s));
-      B.st.reset();
+      launch_kry_residual(s, bt, rt, N, kp, hv, Vb);
+      fetch(1);
+      beta = std::sqrt(hh[0]);
     }
-    {
-      const double rn = std::sqrt(dot(rt, rt));
-      rel = rn / bnorm;
-    }
+    rel = beta / bnorm;
     if (dev) {
       launch_scatter_perm(s, xt, t->d_perm, x, (int)NP, dof);
     } else {
