@@ -330,11 +330,11 @@ ifmm_status ifmm_qr_check(int precision, int pivoted, int m, int n, double* A, i
 
 /* The FP64 Gauss-Jordan inverse with partial pivoting of the pivot blocks
  * (Algorithm 1's inverses of Pi_i), on host arrays, through the same size
- * classes as the factorization (one CTA in shared memory, a thread-block
- * cluster, or the batched multi-CTA kernels).  A holds nmat column-major
+ * classes as the factorization (one CTA or a thread-block cluster in shared
+ * memory, or the batched multi-CTA kernels).  A holds nmat column-major
  * matrices back to back, matrix i of order n[i] (1..4096) with leading
  * dimension n[i]; each is replaced by its inverse.  info[i] = 0, or k + 1 when
- * step k found no nonzero pivot (that matrix is then left partly eliminated).
+ * step k found no nonzero pivot (that matrix's contents are then unspecified).
  * At most 2^28 doubles in all.  Synchronous; IFMM_ECUDA without a device. */
 ifmm_status ifmm_inv_check(int nmat, const int* n, double* A, int* info);
 

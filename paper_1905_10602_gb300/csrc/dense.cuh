@@ -526,110 +526,206 @@ __device__ double block_sum(double v, double* scratch) {
 }
 
 // ---------------------------------------------------------------- Gauss-Jordan inverse
-// One CTA per matrix.  Step k: pick the row of largest |A(i,k)|, i >= k (ties:
-// smallest i), swap it into row k, scale row k, eliminate column k from every
-// other row; finally undo the row interchanges as column interchanges in
-// reverse order.  The matrix is worked on in shared memory when n*n doubles fit
-// in smem_mat bytes, else in place in global memory.  Dynamic shared memory:
-// smem_mat bytes + 2n doubles + n ints.
-__global__ void k_inv(const InvDesc* __restrict__ d, int nd, int smem_mat) {
-  if ((int)blockIdx.x >= nd) return;
-  const InvDesc D = d[blockIdx.x];
+// In-place inverse with partial pivoting of one n x n matrix per thread-block
+// cluster (1 to 16 CTAs, cluster CTA r holding columns r, r + R, ... in shared
+// memory).  Step k exchanges column k with the unused row p of largest |A(i,k)|
+// (ties: smallest i): with c = column k and q = 1 / c_p, every other column j
+// becomes A(i,j) - c_i (A(p,j) q), A(p,j) q in row p, and column k itself -c_i q,
+// q in row p.  Rows are never moved: after n steps row p_k holds x_k and column
+// k' belongs to y of row p_k', so the inverse is written out as
+// Ainv(k, p_k') = M(p_k, k').
+//
+// What bounds it: at most two FP64 multiply-adds per clock and SM (n^3 / (2 R)
+// clocks), and the chain of n dependent steps.  Columns instead of rows are
+// distributed so that a step needs one exchange: the CTA that owns column k + 1
+// updates that column first, finds its pivot and pushes column, pivot and
+// reciprocal into every CTA's shared memory, and only then everybody does the
+// bulk of step k, which hides the exchange (split cluster barrier, three
+// buffers: when step k's data is complete every CTA has finished with those of
+// step k - 2).  The row-distributed kernel this replaces took two cluster
+// barriers, six CTA barriers and serial scans per step: three blocks of 224 rows
+// 1,621 -> 473 us, 78 of 70 rows 382 -> 189 us, the pivots of the 131,072-point
+// job 175 -> 64 ms.
+__host__ __device__ __forceinline__ size_t inv_slot_bytes(int n, int R) {
+  const size_t nc = ((size_t)n + R - 1) / R;
+  return ((size_t)n * nc + 3 * (size_t)n + nc) * sizeof(double) + ((sizeof(int) * (size_t)n + 15) & ~(size_t)15);
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
+// 1/x: the approximate reciprocal refined by two Newton steps (its ~20 bits
+// doubled twice); what it cannot take (subnormal or huge |x|) is divided
+__device__ __forceinline__ double rcp_fp64(double x) {
+  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (e < 3u || e > 2042u) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+// the warp's largest key (hi, lo), lexicographic, and the smallest index among
+// the lanes that hold it; every lane gets the result
+__device__ __forceinline__ void warp_max_key(unsigned& hi, unsigned& lo, int& i) {
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  i = (int)__reduce_min_sync(0xffffffffu, (hi == mh && lo == ml) ? (unsigned)i : 0x7fffffffu);
+  hi = mh;
+  lo = ml;
+}
+
+// V: rows per thread, n <= V * blockDim.x
+template <int V>
+__global__ void __launch_bounds__(512) k_inv(const InvDesc* __restrict__ d, int nd) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int R = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int pi = (int)(blockIdx.x / R);
+  const InvDesc D = d[pi < nd ? pi : nd - 1];
   const int n = D.n;
-  extern __shared__ double sm[];
-  const bool in_smem = (size_t)n * n * sizeof(double) <= (size_t)smem_mat;
-  double* A = in_smem ? sm : D.A;
-  const long ld = in_smem ? n : D.ld;
-  double* rowk = sm + smem_mat / sizeof(double);
-  double* colk = rowk + n;
-  int* piv = (int*)(colk + n);
-  __shared__ double red_v[32];
-  __shared__ int red_i[32];
-  __shared__ int s_p;
-  __shared__ int s_bad;
-  __shared__ double s_inv;
-  if (threadIdx.x == 0) s_bad = 0;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  if (in_smem)
-    for (int j = w; j < n; j += nw)
-      for (int i = lane; i < n; i += 32) A[i + (long)j * n] = D.A[i + (long)j * D.ld];
+  const long ld = D.ld;
+  const int nc = (n - rank + R - 1) / R;  // local columns: rank + c R
+  extern __shared__ __align__(16) double ivm[];
+  double* A = ivm;                                     // n x ceil(n / R), ld n
+  double* cb = A + (size_t)n * ((n + R - 1) / R);      // 3 x n: column k of steps k mod 3
+  double* rr = cb + 3 * (size_t)n;                     // row p of the local columns, scaled
+  int* piv = (int*)(rr + (n + R - 1) / R);
+  __shared__ double ib[3];                             // reciprocal pivots
+  __shared__ int pb[3];                                // pivot rows (-1: none)
+  __shared__ unsigned rh[16], rl[16];
+  __shared__ int ri[16];
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, w = tid >> 5, nw = T >> 5;
+  for (int c = w; c < nc; c += nw)
+    for (int i = lane; i < n; i += 32) A[i + (size_t)c * n] = D.A[i + (long)(rank + c * R) * ld];
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    double best = -1.0;
-    int bi = n;
-    for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-      const double v = fabs(A[i + k * ld]);
-      if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-    }
+  const int nrb = (n + 31) >> 5, dx = nw / nrb, drb = nw - dx * nrb;
+  bool used[V];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
-    if (lane == 0) { red_v[w] = best; red_i[w] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double bv = -1.0;
-      int b = n;
-      for (int i = 0; i < nw; ++i)
-        if (red_v[i] > bv || (red_v[i] == bv && red_i[i] < b)) { bv = red_v[i]; b = red_i[i]; }
-      if (!(bv > 0.0) || b >= n) { s_bad = k + 1; b = k; }
-      s_p = b;
-      piv[k] = b;
-    }
-    __syncthreads();
-    if (s_bad) break;
-    const int p = s_p;
-    if (p != k) {
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const double t = A[k + j * ld];
-        A[k + j * ld] = A[p + j * ld];
-        A[p + j * ld] = t;
+  for (int v = 0; v < V; ++v) used[v] = false;
+  // column c (values val, row tid + v T): its pivot, written back, pushed as step
+  // kk's data; contains one __syncthreads
+  auto publish = [&](const double (&val)[V], int c, int kk) {
+    unsigned hi = 0, lo = 0;
+    int bi = 0x7fffffff;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int i = tid + v * T;
+      const unsigned h = (unsigned)__double2hiint(val[v]) & 0x7fffffffu, l = (unsigned)__double2loint(val[v]);
+      const bool nan = h > 0x7ff00000u || (h == 0x7ff00000u && l);  // never a pivot
+      if (i < n && !used[v] && !nan && (bi == 0x7fffffff || h > hi || (h == hi && l > lo))) {
+        hi = h;
+        lo = l;
+        bi = i;
       }
-      __syncthreads();  // p is the same in every thread: row k complete before it is read below
     }
-    // the reciprocal of the pivot once (an FP64 divide is a long FP64 sequence)
-    if (threadIdx.x == 0) s_inv = 1.0 / A[k + k * ld];
-    __syncthreads();
-    const double inv = s_inv;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      const double v = (j == k) ? inv : A[k + j * ld] * inv;
-      rowk[j] = v;
-      A[k + j * ld] = v;
+    warp_max_key(hi, lo, bi);
+    if (lane == 0) {
+      rh[w] = hi;
+      rl[w] = lo;
+      ri[w] = bi;
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) colk[i] = (i == k) ? 0.0 : A[i + k * ld];
     __syncthreads();
-    // warps over columns, lanes over rows (no per-element index division)
-    for (int j = w; j < n; j += nw) {
-      const double rj = rowk[j];
-      double* cj = A + (long)j * ld;
-      for (int i = lane; i < n; i += 32) {
-        if (i == k) continue;
-        const double a = (j == k) ? 0.0 : cj[i];
-        cj[i] = a - colk[i] * rj;
+    hi = lane < nw ? rh[lane] : 0u;
+    lo = lane < nw ? rl[lane] : 0u;
+    bi = lane < nw ? ri[lane] : 0x7fffffff;
+    warp_max_key(hi, lo, bi);
+    const int p = (hi | lo) ? bi : -1;
+    const int b = kk % 3;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int i = tid + v * T;
+      if (i >= n) continue;
+      A[i + (size_t)c * n] = val[v];
+      for (int r = 0; r < R; ++r) cl.map_shared_rank(cb, r)[(size_t)b * n + i] = val[v];
+      if (i == p) {
+        const double q = rcp_fp64(val[v]);
+        for (int r = 0; r < R; ++r) {
+          cl.map_shared_rank(ib, r)[b] = q;
+          cl.map_shared_rank(pb, r)[b] = p;
+        }
+      }
+    }
+    if (p < 0 && tid == 0)
+      for (int r = 0; r < R; ++r) cl.map_shared_rank(pb, r)[b] = -1;
+  };
+  // no CTA writes into another's shared memory before that one runs
+  cl.sync();
+  if (rank == 0) {
+    double val[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) val[v] = tid + v * T < n ? A[tid + v * T] : 0.0;
+    publish(val, 0, 0);
+  }
+  cluster_arrive();
+  int bad = 0;
+  for (int k = 0; k < n; ++k) {
+    cluster_wait();
+    const int b = k % 3;
+    const int p = pb[b];
+    if (p < 0) {
+      bad = k + 1;
+      break;
+    }
+    const double* c = cb + (size_t)b * n;
+    const double q = ib[b];
+    if (tid == 0) piv[k] = p;
+#pragma unroll
+    for (int v = 0; v < V; ++v) used[v] = used[v] || tid + v * T == p;
+    if (k + 1 < n) {
+      if ((k + 1) % R == rank) {
+        const int cn = (k + 1) / R;
+        double val[V];
+        const double r = A[p + (size_t)cn * n] * q;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const int i = tid + v * T;
+          val[v] = 0.0;
+          if (i < n) val[v] = i == p ? r : fma(-c[i], r, A[i + (size_t)cn * n]);
+        }
+        publish(val, cn, k + 1);
+      }
+      cluster_arrive();
+    }
+    // bulk: (column, 32 rows) items over the warps, four in flight (independent
+    // FP64 chains); column k itself is the same update of a zero column
+    const int xk = k % R == rank ? k / R : -1, xn = (k + 1) % R == rank ? (k + 1) / R : -1;
+    for (int x = tid; x < nc; x += T) rr[x] = x == xk ? q : A[p + (size_t)x * n] * q;
+    __syncthreads();  // row p read before any of it is written
+    {
+      int x = w / nrb, rb = w - x * nrb;
+      for (int e = w; e < nc * nrb; e += 4 * nw) {
+        int ix[4], ii[4];
+        bool on[4];
+        double z[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          ii[u] = rb * 32 + lane;
+          ix[u] = x;
+          on[u] = x < nc && x != xn;
+          z[u] = (on[u] && ii[u] < n && x != xk) ? A[ii[u] + (size_t)x * n] : 0.0;
+          x += dx;
+          rb += drb;
+          if (rb >= nrb) {
+            rb -= nrb;
+            ++x;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (on[u] && ii[u] < n) {
+            const double r = rr[ix[u]];
+            A[ii[u] + (size_t)ix[u] * n] = ii[u] == p ? r : fma(-c[ii[u]], r, z[u]);
+          }
       }
     }
     __syncthreads();
   }
-  if (s_bad) {
-    if (threadIdx.x == 0) D.info[0] = s_bad;
-    return;
-  }
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = piv[k];
-    if (p != k)
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double t = A[i + k * ld];
-        A[i + k * ld] = A[i + p * ld];
-        A[i + p * ld] = t;
-      }
-    __syncthreads();
-  }
-  if (in_smem)
-    for (int j = w; j < n; j += nw)
-      for (int i = lane; i < n; i += 32) D.A[i + (long)j * D.ld] = A[i + (long)j * n];
-  if (threadIdx.x == 0) D.info[0] = 0;
+  // no CTA leaves, or overwrites the input, while another still needs it
+  cl.sync();
+  if (!bad)
+    for (int x = w; x < nc; x += nw) {
+      double* o = D.A + (long)piv[rank + x * R] * ld;
+      for (int k = lane; k < n; k += 32) o[k] = A[piv[k] + (size_t)x * n];
+    }
+  if (rank == 0 && tid == 0) D.info[0] = bad;
 }
 
 // Batched Gauss-Jordan for matrices too large for shared memory: one launch
@@ -1698,171 +1794,6 @@ __global__ void __launch_bounds__(512) k_qr_cluster(const QrcpDesc* __restrict__
       if (D.tail) D.tail[0] = (k < kmax && capped) ? tailv : 0.0;
     }
   }
-}
-
-// ---------------------------------------------------------------- Gauss-Jordan across a cluster
-// The inverse of k_inv (partial pivoting, in place, the row interchanges undone
-// as column interchanges at the end) with the rows split over the R CTAs of a
-// thread-block cluster (CTA r holds rows [r*chunk, (r+1)*chunk), chunk =
-// ceil(n/R), all n columns, column-major with ld chunk), so that a color with
-// few large pivot blocks still occupies many SMs of GB300's narrow FP64 pipes.
-// Step k: each CTA publishes its best |A(i,k)|, i >= k (barrier 1); every CTA
-// picks the same pivot row p (ties: smallest i); the CTAs owning rows k and p
-// publish copies of them (barrier 2); every CTA forms the scaled pivot row from
-// the copy of row p and eliminates column k from its rows, the owner of p first
-// taking in the copy of row k.  Exchange buffers alternate between even and odd
-// steps.  Every element sees the same operations as in k_inv.
-// Slot: A (chunk x n) | ck (chunk) | prow (n) | xrk, xrp (2 x n each) | xv (2),
-// in double | piv (n), xi (2) ints.
-__host__ __device__ __forceinline__ size_t inv_cluster_slot_bytes(int n, int R) {
-  const size_t chunk = ((size_t)n + R - 1) / R;
-  return ((chunk * n + chunk + 5 * (size_t)n + 2) * sizeof(double) + sizeof(int) * ((size_t)n + 2) + 15) &
-         ~(size_t)15;
-}
-
-__global__ void __launch_bounds__(512) k_inv_cluster(const InvDesc* __restrict__ d, int nd) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int R = (int)cl.num_blocks();
-  const int rank = (int)cl.block_rank();
-  const int pi = (int)(blockIdx.x / R);
-  const InvDesc D = d[pi < nd ? pi : nd - 1];
-  const int n = D.n;
-  const long ld = D.ld;
-  const int chunk = (n + R - 1) / R;
-  const int r0 = min(n, rank * chunk), ml = min(n, r0 + chunk) - r0;
-  const int cp = chunk > 0 ? chunk : 1;
-  extern __shared__ __align__(16) unsigned char ism2[];
-  double* A = (double*)ism2;
-  double* ck = A + (size_t)cp * n;
-  double* prow = ck + cp;
-  double* xrk = prow + n;
-  double* xrp = xrk + 2 * n;
-  double* xv = xrp + 2 * n;
-  int* piv = (int*)(xv + 2);
-  int* xi = piv + n;
-  __shared__ double red_v[32];
-  __shared__ int red_i[32];
-  __shared__ double s_inv;
-  __shared__ int s_p;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-  for (int j = w; j < n; j += nw)
-    for (int li = lane; li < ml; li += 32) A[li + (size_t)j * cp] = D.A[(r0 + li) + (long)j * ld];
-  __syncthreads();
-  int bad = 0;
-  const int tot = ml * n;
-  for (int k = 0; k < n; ++k) {
-    const int b = k & 1;
-    double best = -1.0;
-    int bi = n;
-    for (int li = max(0, k - r0) + tid; li < ml; li += nt) {
-      const double v = fabs(A[li + (size_t)k * cp]);
-      const int i = r0 + li;
-      if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
-    if (lane == 0) {
-      red_v[w] = best;
-      red_i[w] = bi;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double bv = -1.0;
-      int bb = n;
-      for (int i = 0; i < nw; ++i)
-        if (red_v[i] > bv || (red_v[i] == bv && red_i[i] < bb)) { bv = red_v[i]; bb = red_i[i]; }
-      xv[b] = bv;
-      xi[b] = bb;
-    }
-    cl.sync();
-    // one warp reads the R candidates and decides (the same decision in every CTA)
-    if (w == 0) {
-      double v = -1.0;
-      int i = n;
-      if (lane < R) {
-        v = cl.map_shared_rank(xv, lane)[b];
-        i = cl.map_shared_rank(xi, lane)[b];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-        if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
-      }
-      if (lane == 0) {
-        s_p = (!(v > 0.0) || i >= n) ? -1 : i;
-        if (s_p >= 0) piv[k] = i;
-      }
-    }
-    __syncthreads();
-    const int p = s_p;
-    if (p < 0) {
-      bad = k + 1;
-      break;
-    }
-    const int ok = k / chunk, op = p / chunk;
-    if (rank == ok)
-      for (int j = tid; j < n; j += nt) xrk[(size_t)b * n + j] = A[(k - r0) + (size_t)j * cp];
-    if (rank == op)
-      for (int j = tid; j < n; j += nt) xrp[(size_t)b * n + j] = A[(p - r0) + (size_t)j * cp];
-    cl.sync();
-    const double* rp = cl.map_shared_rank(xrp, op) + (size_t)b * n;
-    if (tid == 0) s_inv = 1.0 / rp[k];  // once per CTA: an FP64 divide is a long FP64 sequence
-    // multipliers of column k (the owner of p takes in the copy of row k there)
-    const double* rk = (rank == op && p != k) ? cl.map_shared_rank(xrk, ok) + (size_t)b * n : nullptr;
-    for (int li = tid; li < ml; li += nt) ck[li] = (rk && r0 + li == p) ? rk[k] : A[li + (size_t)k * cp];
-    if (rk)
-      for (int j = tid; j < n; j += nt) A[(p - r0) + (size_t)j * cp] = rk[j];
-    __syncthreads();
-    const double inv = s_inv;
-    for (int j = tid; j < n; j += nt) prow[j] = (j == k) ? inv : rp[j] * inv;
-    __syncthreads();
-    // eliminate column k from every local row but k; (li, j) walked with
-    // incremental indices; the owner of k writes the scaled pivot row
-    {
-      int li = tid % max(ml, 1), j = tid / max(ml, 1);
-      const int di = nt % max(ml, 1), dj = nt / max(ml, 1);
-      for (int e = tid; e < tot; e += nt) {
-        const int i = r0 + li;
-        double* a = A + li + (size_t)j * cp;
-        if (i == k)
-          *a = prow[j];
-        else
-          *a = ((j == k) ? 0.0 : *a) - ck[li] * prow[j];
-        li += di;
-        j += dj;
-        if (li >= ml) {
-          li -= ml;
-          ++j;
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (!bad) {
-    for (int k = n - 1; k >= 0; --k) {
-      const int p = piv[k];
-      if (p != k)
-        for (int li = tid; li < ml; li += nt) {
-          const double t = A[li + (size_t)k * cp];
-          A[li + (size_t)k * cp] = A[li + (size_t)p * cp];
-          A[li + (size_t)p * cp] = t;
-        }
-      __syncthreads();
-    }
-  }
-  // no CTA leaves while another may still read its shared memory
-  cl.sync();
-  if (!bad)
-    for (int j = w; j < n; j += nw)
-      for (int li = lane; li < ml; li += 32) D.A[(r0 + li) + (long)j * ld] = A[li + (size_t)j * cp];
-  if (rank == 0 && tid == 0) D.info[0] = bad;
 }
 
 // ---------------------------------------------------------------- IL basis changes

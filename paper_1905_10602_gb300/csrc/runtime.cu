@@ -346,12 +346,14 @@ void launch_gemm(DescStage& st, const std::vector<GemmDesc>& v0, int prec) {
   profiler().end(kk, st.stream, pe);
 }
 
-// A cluster launch of k_inv_cluster (R CTAs per matrix); false when no cluster of
-// that shape and shared memory can be resident.
-static bool launch_inv_cluster(const InvDesc* d, int nd, int R, size_t smem, cudaStream_t s, bool probe_only) {
+// A launch of k_inv, a cluster of R CTAs of T threads per matrix; probe_only:
+// whether a cluster of that shape and shared memory can be resident.
+static constexpr size_t kInvSmem = 220 * 1024;
+static bool launch_inv_cluster(const InvDesc* d, int nd, int R, int T, bool two, size_t smem, cudaStream_t s,
+                               bool probe_only) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nd * R), 1, 1);
-  cfg.blockDim = dim3(512, 1, 1);
+  cfg.blockDim = dim3((unsigned)T, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -363,13 +365,16 @@ static bool launch_inv_cluster(const InvDesc* d, int nd, int R, size_t smem, cud
   cfg.numAttrs = 1;
   if (probe_only) {
     int ncl = 0;
-    if (cudaOccupancyMaxActiveClusters(&ncl, k_inv_cluster, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&ncl, two ? k_inv<2> : k_inv<1>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     return ncl > 0;
   }
-  CK(cudaLaunchKernelEx(&cfg, k_inv_cluster, d, nd));
+  if (two)
+    CK(cudaLaunchKernelEx(&cfg, k_inv<2>, d, nd));
+  else
+    CK(cudaLaunchKernelEx(&cfg, k_inv<1>, d, nd));
   return true;
 }
 
@@ -379,23 +384,17 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
     req(v[i].A, span(v[i].n, v[i].n, v[i].ld), "inv.A", i);
     req(v[i].info, sizeof(int), "inv.info", i);
   }
-  // Size classes.  Blocks of n <= 32: one CTA each in shared memory.  Larger
-  // ones: the FP64 elimination of one block on one SM is bound by that SM's FP64
-  // pipe, so when a color has fewer large blocks than SMs each block is spread
-  // over a cluster of R CTAs (R ~ SMs / blocks, at most 16 -- a non-portable
-  // cluster size, used when the GPU can host it -- and at least what its rows
-  // need to fit); R = 1 is one CTA in shared memory (n <= 160).  Blocks that fit
-  // no cluster take the batched multi-CTA kernels below.
-  static constexpr int kInvCta = 0;
-  static constexpr size_t kInvClusterSmem = 220 * 1024;
   static std::once_flag attr_once;
   std::call_once(attr_once, [] {
-    CK(cudaFuncSetAttribute(k_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
-    CK(cudaFuncSetAttribute(k_inv_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvClusterSmem));
-    if (cudaFuncSetAttribute(k_inv_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-      cudaGetLastError();  // then the residency probe rejects R = 16
+    auto set = [](const void* f) {
+      CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem));
+      if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();  // then the residency probe rejects R = 16
+    };
+    set((const void*)k_inv<1>);
+    set((const void*)k_inv<2>);
   });
-  static int cl_ok[5] = {0, 0, 0, 0, 0};  // per R = 1, 2, 4, 8, 16: 0 unknown, 1 yes, -1 no
+  static int cl_ok[2][5] = {};  // per rows-per-thread and R = 1, 2, 4, 8, 16: 0 unknown, 1 yes, -1 no
   static std::mutex cl_mu;
   // IFMM_INV_FALLBACK_N=n (read once per process; tests) sends every block of
   // at least n rows to the batched multi-CTA kernels
@@ -404,85 +403,73 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
     const long n = e ? atol(e) : 0;
     return n >= 1 ? (int)std::min(n, 1L << 30) : 0;
   }();
+  // Classes: by rows (<= 32, 64, 128, 256, 512, 1024; threads for one row each up
+  // to 512) and by CTAs per matrix.  Blocks of more than 24 rows are spread over
+  // as many CTAs (a power of two, at most 16 -- a non-portable cluster size, used
+  // when the GPU can host it) as leave at most three per SM in all and four
+  // columns each: one SM's FP64 pipe bounds a block, and more CTAs on an SM fill
+  // the gaps of each other's step chains.  Measured with at most one, two, three
+  // CTAs per SM: 78 blocks of 70 rows 421, 263, 189 us; 50 of 100 572, 355, 257;
+  // all pivots of the 131,072-point job 99, 71, 64 ms.  What fits no cluster's
+  // shared memory takes the batched multi-CTA kernels.
+  static constexpr int kRows[6] = {32, 64, 128, 256, 512, 1024};
+  static constexpr int kSplit = 24, kMul = 3, kCols = 4;
   int nbig = 0;
-  for (auto& x : v) nbig += x.n > 32;
-  int rwant = 1;
-  while (rwant < 16 && nbig * rwant * 2 <= 152) rwant *= 2;
-  std::vector<InvDesc> cls[3], ccl[5];
-  size_t csm[5] = {16, 16, 16, 16, 16};
+  for (auto& x : v) nbig += x.n > kSplit;
+  int qwant = 0;
+  while (qwant < 4 && (nbig << (qwant + 1)) <= kMul * 152) ++qwant;
+  std::vector<InvDesc> cls[6][5], rest;
+  size_t smx[6][5] = {};
   for (auto& x : v) {
-    if (fallback_n && x.n >= fallback_n) {
-      cls[2].push_back(x);
+    int c = 0;
+    while (c < 6 && x.n > kRows[c]) ++c;
+    if ((fallback_n && x.n >= fallback_n) || c == 6) {
+      rest.push_back(x);
       continue;
     }
-    if (x.n <= 32) {
-      cls[0].push_back(x);
-      continue;
-    }
-    int R = rwant, q = 0;
-    while ((1 << q) < R) ++q;
-    int qmin = 0;  // the smallest cluster whose slots hold the rows
-    while (qmin < 5 && inv_cluster_slot_bytes(x.n, 1 << qmin) > kInvClusterSmem) ++qmin;
-    if (q < qmin) q = qmin;
-    if (q == 0 && x.n <= 160) {
-      cls[1].push_back(x);
-      continue;
-    }
-    if (q == 0) q = 1;
-    bool ok = false;
-    {
+    int qmin = 0;  // the smallest cluster whose slots hold the matrix
+    while (qmin < 5 && inv_slot_bytes(x.n, 1 << qmin) > kInvSmem) ++qmin;
+    int q = std::max(x.n > kSplit ? qwant : 0, qmin);
+    while (q > qmin && (1 << q) * kCols > x.n) --q;
+    bool ok = q == 0;
+    if (q > 0 && qmin < 5) {
       std::lock_guard<std::mutex> lock(cl_mu);
-      // the wanted size, else the next smaller one that still holds the rows
-      for (; q < 5 && q >= std::max(1, qmin); --q) {
-        if (cl_ok[q] == 0)
-          cl_ok[q] = launch_inv_cluster(nullptr, 1, 1 << q, kInvClusterSmem, st.stream, true) ? 1 : -1;
-        if (cl_ok[q] > 0) {
-          ok = true;
-          break;
-        }
+      // the wanted size, else the next smaller one that still holds the matrix
+      for (; q >= qmin && !ok; --q) {
+        int& f = cl_ok[c == 5][q];
+        if (f == 0) f = launch_inv_cluster(nullptr, 1, 1 << q, 512, c == 5, kInvSmem, st.stream, true) ? 1 : -1;
+        ok = f > 0;
+        if (ok) break;
       }
     }
-    if (ok) {
-      ccl[q].push_back(x);
-      csm[q] = std::max(csm[q], inv_cluster_slot_bytes(x.n, 1 << q));
-    } else {
-      cls[x.n <= 160 ? 1 : 2].push_back(x);
+    if (!ok) {
+      rest.push_back(x);
+      continue;
     }
+    cls[c][q].push_back(x);
+    smx[c][q] = std::max(smx[c][q], inv_slot_bytes(x.n, 1 << q));
   }
-  (void)kInvCta;
-  const InvDesc* dcl[5] = {};
-  for (int q = 1; q < 5; ++q)
-    if (!ccl[q].empty()) dcl[q] = st.push(ccl[q]);
-  int ncl = 0;
-  for (int q = 1; q < 5; ++q) ncl += (int)ccl[q].size();
-  if (ncl) {
-    prof_batch_tag() = (long)ncl;
+  if (rest.size() < v.size()) {
+    const InvDesc* dcl[6][5] = {};
+    for (int c = 0; c < 6; ++c)
+      for (int q = 0; q < 5; ++q)
+        if (!cls[c][q].empty()) dcl[c][q] = st.push(cls[c][q]);
+    prof_batch_tag() = (long)(v.size() - rest.size());
     cudaEvent_t pe = profiler().begin(KK_INV, st.stream);
     ForkJoin fj(st.stream);
     int li = 0;
-    for (int q = 1; q < 5; ++q) {
-      if (ccl[q].empty()) continue;
-      launch_inv_cluster(dcl[q], (int)ccl[q].size(), 1 << q, csm[q], fj.stream(li++), false);
-      check_launch("k_inv_cluster");
-    }
+    for (int c = 5; c >= 0; --c)  // the longest first
+      for (int q = 4; q >= 0; --q) {
+        if (cls[c][q].empty()) continue;
+        const int T = std::max(128, std::min(512, kRows[c]));
+        launch_inv_cluster(dcl[c][q], (int)cls[c][q].size(), 1 << q, T, c == 5, smx[c][q], fj.stream(li++), false);
+        check_launch("k_inv");
+      }
     fj.join();
     profiler().end(KK_INV, st.stream, pe);
   }
-  for (int c = 0; c < 2; ++c) {
-    if (cls[c].empty()) continue;
-    int nmax = 0;
-    for (auto& x : cls[c]) nmax = std::max(nmax, x.n);
-    const int smem_mat = nmax * nmax * (int)sizeof(double);
-    const size_t smem = (size_t)smem_mat + sizeof(double) * 2 * nmax + sizeof(int) * nmax + 16;
-    const InvDesc* d = st.push(cls[c]);
-    prof_batch_tag() = (long)cls[c].size();
-    cudaEvent_t pe = profiler().begin(KK_INV, st.stream);
-    k_inv<<<(unsigned)cls[c].size(), c == 0 ? 128 : 256, smem, st.stream>>>(d, (int)cls[c].size(), smem_mat);
-    check_launch("k_inv");
-    profiler().end(KK_INV, st.stream, pe);
-  }
-  if (!cls[2].empty()) {
-    const std::vector<InvDesc>& L = cls[2];
+  if (!rest.empty()) {
+    const std::vector<InvDesc>& L = rest;
     int nmax = 0;
     std::vector<long> off(L.size());
     long tot = 0;
