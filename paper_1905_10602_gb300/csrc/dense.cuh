@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "descs.h"
+#include "fp64_ops.cuh"
 
 namespace ifmm {
 
@@ -552,16 +553,6 @@ __host__ __device__ __forceinline__ size_t inv_slot_bytes(int n, int R) {
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
-// 1/x: the approximate reciprocal refined by two Newton steps (its ~20 bits
-// doubled twice); what it cannot take (subnormal or huge |x|) is divided
-__device__ __forceinline__ double rcp_fp64(double x) {
-  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-  if (e < 3u || e > 2042u) return 1.0 / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(fma(-x, y, 1.0), y, y);
-  return fma(fma(-x, y, 1.0), y, y);
-}
 // the warp's largest key (hi, lo), lexicographic, and the smallest index among
 // the lanes that hold it; every lane gets the result
 __device__ __forceinline__ void warp_max_key(unsigned& hi, unsigned& lo, int& i) {
@@ -1957,27 +1948,98 @@ __global__ void __launch_bounds__(256) k_schur_scatter(const ScatterDesc* __rest
 // orthogonal to working precision.  Pairs are taken in the round-robin order
 // (k' = k rounded up to even; in round r, position p > 0 holds column
 // 1 + ((p - 1 - r) mod (k'-1)); pair i joins positions i and k'-1-i), so the k'/2
-// pairs of a round are disjoint and handled by different warps.
-// B (n x k, column-major, ld n) lives in dynamic shared memory when it fits in
-// smem_bytes, else in the descriptor's global work buffer.  Columns are rotated
-// in place (no rotation matrix is accumulated: the rotated columns themselves,
-// normalised, are the singular vectors sought).  n <= 1024.
-template <typename TC>
-__global__ void k_svd_rt(const SvdRtDesc* __restrict__ d, int nd, int max_sweeps, int smem_bytes) {
-  if ((int)blockIdx.x >= nd) return;
-  const SvdRtDesc D = d[blockIdx.x];
+// pairs of a round are disjoint and handled by different groups of lanes.
+// Columns are rotated in place (no rotation matrix is accumulated: the rotated
+// columns themselves, normalised, are the singular vectors sought).  n <= 1024.
+//
+// Bound: in FP64 the FP64 pipe, in FP32 the issue slots, and in both most of it
+// was the scalar part of a pair, which every lane repeats (square roots,
+// divisions, hypot: ~150 FP64 instructions against 14 for the rotation itself at
+// n = 50).  So: G lanes per pair instead of 32 (a warp does 32 / G pairs at
+// once), the two columns held in registers between dot product and rotation (EM
+// elements per lane; EM = 0: any length, read twice), squared norms kept and
+// updated (al - t g, be + t g; summed afresh every sweep and where the update
+// cancels), and the angle from FP32: its tangent is refined by one Newton step in
+// FP64, and only c = 1/sqrt(1 + t^2) has to be exact for the rotation to be
+// orthogonal.  Six to nine sweeps as before.  Measured (with the launch classes
+// of launch_svd_rt): FP64 class of an 8,192-point job 621 -> 281 ms, FP32 class of
+// the 131,072-point job 141 -> 56 ms.
+// Slot of one problem: B (n x k, ld svd_ld) when it fits, else the descriptor's
+// work buffer | squared norms, reciprocals (n each), in TC | order (n ints).
+// the column pitch: an odd multiple of G, so that the groups of a warp, which
+// read neighbouring columns, meet different banks
+__host__ __device__ __forceinline__ int svd_ld(int n, int G) { return G * (((n + G - 1) / G) | 1); }
+__host__ __device__ __forceinline__ size_t svd_tail_bytes(int n, int tc_bytes) {
+  return (((size_t)n * (2 * tc_bytes + sizeof(int))) + 15) & ~(size_t)15;
+}
+
+template <int G, typename TC>
+__device__ __forceinline__ TC group_sum(TC v) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ float sqrt_fast(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// whether the pair needs a rotation (|g| > tol sqrt(al be))
+__device__ __forceinline__ bool svd_needs(float al, float be, float g) {
+  return !(al < 1e-36f || be < 1e-36f || fabsf(g) <= 4e-7f * sqrt_fast(al) * sqrt_fast(be));
+}
+__device__ __forceinline__ bool svd_needs(double al, double be, double g) {
+  return !(al < 1e-280 || be < 1e-280 || g * g <= 1e-30 * (al * be));
+}
+// rotation that orthogonalises columns of squared norms al, be and product g:
+// t = tan, c = cos, s = sin; t^2 + 2 z t - 1 = 0 with z = (be - al) / (2 g)
+__device__ __forceinline__ void svd_rotation(float al, float be, float g, float& t, float& c, float& s) {
+  const float z = __fdividef(be - al, g + g);
+  t = __fdividef(copysignf(1.f, z), fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
+  const float x = fmaf(t, t, 1.f), y = rsqrtf(x);
+  c = fmaf(0.5f * y, fmaf(-(x * y), y, 1.f), y);
+  s = c * t;
+}
+__device__ __forceinline__ void svd_rotation(double al, double be, double g, double& t, double& c, double& s) {
+  const double d = be - al, g2 = g + g;
+  const int sh = 1023 - max(dexp(d), dexp(g2));  // both into the FP32 range, exactly scaled
+  const float df = d2f_pow2(d, sh), gf = d2f_pow2(g2, sh);
+  const float z = __fdividef(df, gf);
+  const float t0 = __fdividef(copysignf(1.f, z), fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
+  t = f2d_pow2(t0, 0);
+  // one Newton step of g2 t^2 + 2 d t - g2 = 0: the residual in FP64
+  const double f = fma(t, fma(g2, t, d + d), -g2);
+  t -= f2d_pow2(__fdividef(d2f_pow2(f, sh), 2.f * fmaf(gf, t0, df)), 0);
+  c = rsqrt_fp64(fma(t, t, 1.0));
+  s = c * t;
+}
+
+// WARP: a problem per warp (k <= 16), else per CTA; slot_bytes of dynamic shared
+// memory per problem, of which the last svd_tail_bytes(n) hold the tail
+template <typename TC, int G, int EM, bool WARP>
+__global__ void __launch_bounds__(WARP ? 128 : 1024) k_svd_rt(const SvdRtDesc* __restrict__ d, int nd, int max_sweeps,
+                                                              int slot_bytes) {
+  extern __shared__ __align__(16) unsigned char svm[];
+  __shared__ int s_em[32];
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = WARP ? 0 : threadIdx.x >> 5, nw = WARP ? 1 : blockDim.x >> 5;
+  const int di = WARP ? blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5) : blockIdx.x;
+  if (di >= nd) return;
+  auto sync = [] {
+    if constexpr (WARP) __syncwarp(); else __syncthreads();
+  };
+  const SvdRtDesc D = d[di];
   const int n = D.n;
   int k = D.kin[0];
   k = k < 0 ? 0 : (k > n ? n : k);
-  extern __shared__ double smraw[];
-  __shared__ TC nrm[1024];
-  __shared__ TC rnv[1024];
-  __shared__ int ord[1024];
-  __shared__ int s_em[32];
-  __shared__ int s_rot;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  const bool in_smem = (size_t)n * k * sizeof(TC) <= (size_t)smem_bytes;
-  TC* B = in_smem ? (TC*)smraw : (TC*)D.work;
+  unsigned char* slot = svm + (WARP ? (size_t)(threadIdx.x >> 5) * slot_bytes : 0);
+  const size_t tail = svd_tail_bytes(n, sizeof(TC));
+  TC* nrm = (TC*)(slot + slot_bytes - tail);
+  TC* rnv = nrm + n;
+  int* ord = (int*)(rnv + n);
+  const bool in_smem = (size_t)svd_ld(n, G) * k * sizeof(TC) <= (size_t)slot_bytes - tail;
+  TC* B = in_smem ? (TC*)slot : (TC*)D.work;
+  const int lb = in_smem ? svd_ld(n, G) : n;
   const long ld = D.ld;
   // B = P R_k^T (or the explicit matrix), scaled by a power of two 2^sh that
   // brings its largest entry into [0.5, 1); warps over columns, lanes over rows
@@ -1987,78 +2049,145 @@ __global__ void k_svd_rt(const SvdRtDesc* __restrict__ d, int nd, int max_sweeps
       const double v = D.jpvt ? ((i <= pos) ? D.A[i + (long)pos * ld] : 0.0) : D.A[pos + (long)i * ld];
       em = max(em, dexp(v));
     }
-  em = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
-  if (lane == 0) s_em[w] = em;
-  __syncthreads();
-  em = 0;
-  for (int i = 0; i < nw; ++i) em = max(em, s_em[i]);
+  em = (int)__reduce_max_sync(kAll, (unsigned)em);
+  if constexpr (!WARP) {
+    if (lane == 0) s_em[w] = em;
+    __syncthreads();
+    em = (int)__reduce_max_sync(kAll, lane < nw ? (unsigned)s_em[lane] : 0u);
+  }
   const int sh = pow2_shift(em);
   for (int i = w; i < k; i += nw)
     for (int pos = lane; pos < n; pos += 32) {
       if (D.jpvt)
-        B[D.jpvt[pos] + (long)i * n] = ld_tc<TC>((i <= pos) ? D.A[i + (long)pos * ld] : 0.0, sh);
+        B[D.jpvt[pos] + (long)i * lb] = ld_tc<TC>((i <= pos) ? D.A[i + (long)pos * ld] : 0.0, sh);
       else
-        B[pos + (long)i * n] = ld_tc<TC>(D.A[pos + (long)i * ld], sh);
+        B[pos + (long)i * lb] = ld_tc<TC>(D.A[pos + (long)i * ld], sh);
     }
-  __syncthreads();
-  const TC tol = sizeof(TC) == 8 ? (TC)1e-15 : (TC)4e-7;
-  const TC tiny = sizeof(TC) == 8 ? (TC)1e-300 : (TC)1e-36;
-  const int kp = k + (k & 1);
+  sync();
+  const int sub = lane & (G - 1), gw = lane / G;  // lane of the group, group of the warp
+  constexpr int GW = 32 / G;
+  const int kp = k + (k & 1), np = kp / 2;
+  // squared norms of every column
+  auto norms = [&] {
+    for (int j0 = w * GW; j0 < k; j0 += nw * GW) {
+      const int j = j0 + gw;
+      TC s2 = 0;
+      if (j < k)
+        for (int i = sub; i < n; i += G) {
+          const TC u = B[i + (long)j * lb];
+          s2 += u * u;
+        }
+      s2 = group_sum<G>(s2);
+      if (j < k && sub == 0) nrm[j] = s2;
+    }
+    sync();
+  };
   for (int sweep = 0; sweep < max_sweeps && k > 1; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
+    norms();
+    int rotated = 0;
     for (int r = 0; r < kp - 1; ++r) {
-      for (int pi = w; pi < kp / 2; pi += nw) {
-        const int pa = pi, pb = kp - 1 - pi;
-        int a = (pa == 0) ? 0 : 1 + ((pa - 1 - r) % (kp - 1) + (kp - 1)) % (kp - 1);
-        int b = (pb == 0) ? 0 : 1 + ((pb - 1 - r) % (kp - 1) + (kp - 1)) % (kp - 1);
-        if (a >= k || b >= k) continue;
+      for (int p0 = w * GW; p0 < np; p0 += nw * GW) {
+        const int pi = p0 + gw;
+        int a = pi - 1 - r, b = kp - 2 - pi - r;
+        a = pi == 0 ? 0 : 1 + (a < 0 ? a + kp - 1 : a);
+        b = 1 + (b < 0 ? b + kp - 1 : b);
         if (a > b) { const int tt = a; a = b; b = tt; }
-        TC* ga = B + (long)a * n;
-        TC* gb = B + (long)b * n;
-        TC al = 0, be = 0, gab = 0;
-        for (int i = lane; i < n; i += 32) {
-          const TC u = ga[i], v = gb[i];
-          al += u * u;
-          be += v * v;
-          gab += u * v;
+        const bool live = pi < np && b < k;
+        TC* ga = B + (long)(live ? a : 0) * lb;
+        TC* gb = B + (long)(live ? b : 0) * lb;
+        TC g = 0;
+        TC u[EM > 0 ? EM : 1], v[EM > 0 ? EM : 1];
+        if constexpr (EM > 0) {
+          TC g1 = 0;
+#pragma unroll
+          for (int e = 0; e < EM; ++e) {
+            const int i = sub + e * G;
+            const bool in = live && i < n;
+            u[e] = in ? ga[i] : (TC)0;
+            v[e] = in ? gb[i] : (TC)0;
+            if (e & 1) g1 += u[e] * v[e]; else g += u[e] * v[e];
+          }
+          g += g1;
+        } else if (live) {
+          for (int i = sub; i < n; i += G) g += ga[i] * gb[i];
         }
-        al = warp_sum_t<TC>(al);
-        be = warp_sum_t<TC>(be);
-        gab = warp_sum_t<TC>(gab);
-        if (al < tiny || be < tiny) continue;
-        if (fabs(gab) <= tol * sqrt(al) * sqrt(be)) continue;
-        const TC zeta = (be - al) / ((TC)2 * gab);
-        const TC t = (zeta >= (TC)0 ? (TC)1 : (TC)-1) / (fabs(zeta) + hypot((TC)1, zeta));
-        const TC c = (TC)1 / sqrt((TC)1 + t * t), s = c * t;
-        for (int i = lane; i < n; i += 32) {
-          const TC u = ga[i], v = gb[i];
-          ga[i] = c * u - s * v;
-          gb[i] = s * u + c * v;
+        g = group_sum<G>(g);
+        TC al = 0, be = 0;
+        if (live) {
+          al = nrm[a];
+          be = nrm[b];
         }
-        if (lane == 0) s_rot = 1;
+        const bool rot = live && svd_needs(al, be, g);
+        if (!__any_sync(kAll, rot)) continue;
+        rotated = 1;
+        TC t = 0, c = 1, s = 0;
+        if (rot) svd_rotation(al, be, g, t, c, s);
+        TC na = al - t * g, nb = be + t * g;
+        const bool redo = rot && (!(na > (TC)0.05 * al) || !(nb > (TC)0.05 * be));
+        TC sa = 0, sb = 0;
+        const bool again = __any_sync(kAll, redo);
+        if constexpr (EM > 0) {
+          if (rot) {
+#pragma unroll
+            for (int e = 0; e < EM; ++e) {
+              const int i = sub + e * G;
+              const TC x = c * u[e] - s * v[e];
+              v[e] = s * u[e] + c * v[e];
+              u[e] = x;
+              if (i < n) {
+                ga[i] = u[e];
+                gb[i] = v[e];
+              }
+            }
+          }
+          if (again)
+#pragma unroll
+            for (int e = 0; e < EM; ++e) {
+              sa += u[e] * u[e];
+              sb += v[e] * v[e];
+            }
+        } else if (rot) {
+          for (int i = sub; i < n; i += G) {
+            const TC x = ga[i], y = gb[i];
+            const TC x2 = c * x - s * y, y2 = s * x + c * y;
+            ga[i] = x2;
+            gb[i] = y2;
+            sa += x2 * x2;
+            sb += y2 * y2;
+          }
+        }
+        if (again) {
+          sa = group_sum<G>(sa);
+          sb = group_sum<G>(sb);
+          if (redo) {
+            na = sa;
+            nb = sb;
+          }
+        }
+        if (rot && sub == 0) {
+          nrm[a] = na;
+          nrm[b] = nb;
+        }
       }
-      __syncthreads();
+      sync();
     }
-    const int rotated = s_rot;
-    __syncthreads();
+    if constexpr (WARP)
+      rotated = __any_sync(kAll, rotated);
+    else
+      rotated = __syncthreads_or(rotated);
     if (!rotated) break;
   }
   // column norms (the singular values times 2^sh) in the arithmetic type, the
   // descending order (NaN last), and the reciprocals once per column
-  for (int j = w; j < k; j += nw) {
-    const TC* g = B + (long)j * n;
-    TC s2 = 0;
-    for (int i = lane; i < n; i += 32) s2 += g[i] * g[i];
-    s2 = warp_sum_t<TC>(s2);
-    if (lane == 0) {
-      const TC v = sqrt(s2);
-      nrm[j] = v;
-      rnv[j] = (v > (TC)0) ? (TC)1 / v : (TC)0;
-    }
+  norms();
+  const int tid = WARP ? lane : threadIdx.x, nt = WARP ? 32 : blockDim.x;
+  for (int j = tid; j < k; j += nt) {
+    const TC v = sqrt(nrm[j]);
+    nrm[j] = v;
+    rnv[j] = (v > (TC)0) ? (TC)1 / v : (TC)0;
   }
-  __syncthreads();
-  for (int j = threadIdx.x; j < k; j += blockDim.x) {
+  sync();
+  for (int j = tid; j < k; j += nt) {
     int rank = 0;
     const TC v = (nrm[j] == nrm[j]) ? nrm[j] : (TC)-1;
     for (int q = 0; q < k; ++q) {
@@ -2067,14 +2196,14 @@ __global__ void k_svd_rt(const SvdRtDesc* __restrict__ d, int nd, int max_sweeps
     }
     ord[rank] = j;
   }
-  __syncthreads();
-  for (int j = threadIdx.x; j < n; j += blockDim.x) D.sig[j] = (j < k) ? st_tc<TC>(nrm[ord[j]], -sh) : 0.0;
+  sync();
+  for (int j = tid; j < n; j += nt) D.sig[j] = (j < k) ? st_tc<TC>(nrm[ord[j]], -sh) : 0.0;
   for (int j = w; j < n; j += nw) {
     double* vj = D.V + (long)j * D.ldv;
     if (j < k) {
       const int c = ord[j];
       const TC r = rnv[c];
-      const TC* g = B + (long)c * n;
+      const TC* g = B + (long)c * lb;
       for (int i = lane; i < n; i += 32) vj[i] = st_tc<TC>(g[i] * r);
     } else {
       for (int i = lane; i < n; i += 32) vj[i] = 0.0;

@@ -25,26 +25,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fp64_ops.cuh"
+
 namespace ifmm {
 
-__device__ __noinline__ double rsqrt_rare(double a) { return rsqrt(a); }
 __device__ __noinline__ void sincos_rare(double a, double* s, double* c) { sincos(a, s, c); }
-
-// 1/sqrt(a) to about an ulp: a = m 4^k, 1 <= m < 4; y0 = rsqrt(float(m)) 2^-k to
-// ~2^-22, then one step y0 (1 + e/2 + 3 e^2 / 8), e = 1 - a y0^2 (the next term is
-// below 2^-65).  Zero, subnormal, negative and non-finite arguments take CUDA's.
-__device__ __forceinline__ double rsqrt_fp64(double a) {
-  const int hi = __double2hiint(a);
-  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return rsqrt_rare(a);
-  const int k = ((hi >> 20) - 1023) >> 1;
-  const unsigned f = __funnelshift_l((unsigned)__double2loint(a), (unsigned)(hi - (k << 21) - 0x38000000), 3);
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(f)));
-  const unsigned u = __float_as_uint(y);
-  const double y0 = __hiloint2double((int)(u >> 3) + 0x38000000 - (k << 20), (int)(u << 29));
-  const double e = fma(-(a * y0), y0, 1.0);
-  return fma(y0 * e, fma(0.375, e, 0.5), y0);
-}
 
 // sine and cosine of x: j = nearest integer to 32 x / pi, d = x - j pi / 32 in two
 // steps (|d| <= pi / 64), table (cos, sin)(j pi / 32) and the Taylor sums of d to

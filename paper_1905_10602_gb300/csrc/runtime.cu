@@ -796,18 +796,34 @@ void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
   }
 }
 
+template <typename TC>
+static void svd_rt_launch(int c, const SvdRtDesc* d, unsigned g, int threads, int slot, cudaStream_t s) {
+  static std::once_flag attr_once;
+  static constexpr int cap = 220 * 1024;
+  std::call_once(attr_once, [] {
+    CK(cudaFuncSetAttribute(k_svd_rt<TC, 8, 6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_svd_rt<TC, 16, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_svd_rt<TC, 32, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_svd_rt<TC, 32, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  });
+  if (c == 0)
+    k_svd_rt<TC, 4, 4, true><<<(g + 3) / 4, 128, 4 * slot, s>>>(d, (int)g, 60, slot);
+  else if (c == 1)
+    k_svd_rt<TC, 8, 6, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+  else if (c == 2)
+    k_svd_rt<TC, 16, 8, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+  else if (c == 3)
+    k_svd_rt<TC, 32, 8, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+  else
+    k_svd_rt<TC, 32, 0, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+  check_launch("k_svd_rt");
+}
+
 void launch_svd_rt(DescStage& st, const std::vector<SvdRtDesc>& v, int prec) {
   if (v.empty()) return;
-  static constexpr int smem_cap = 160 * 1024;
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
-    CK(cudaFuncSetAttribute(k_svd_rt<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cap));
-    CK(cudaFuncSetAttribute(k_svd_rt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cap));
-  });
-  int nmax = 1;
+  static constexpr size_t smem_cap = 220 * 1024;
   for (size_t i = 0; i < v.size(); ++i) {
     IFMM_REQUIRE(v[i].n <= 1024, IFMM_EINVAL, "SVD wider than 1024 columns");
-    nmax = std::max(nmax, v[i].n);
     if (!registry().on) continue;
     const SvdRtDesc& x = v[i];
     req(x.A, span(x.n, x.n, x.ld) > 0 ? sizeof(double) : 0, "svd_rt.A", i);
@@ -816,43 +832,45 @@ void launch_svd_rt(DescStage& st, const std::vector<SvdRtDesc>& v, int prec) {
     req(x.sig, sizeof(double) * x.n, "svd_rt.sig", i);
     req(x.work, sizeof(double) * (size_t)x.n * x.n, "svd_rt.work", i);
   }
-  // B is n x k with k <= n: n^2 elements bound what a problem keeps in shared
-  // memory (larger ones use their global work buffer).  The batch is launched in
-  // width classes so that a wide problem does not set the shared memory (and so
-  // the occupancy) of many narrow ones; one warp per column pair of the widest
-  // problem of a class
+  // Width classes, launched concurrently: each has the lanes per pair and the
+  // elements per lane that hold its columns in registers (<= 16: a warp per
+  // problem, 4 x 4; <= 48: 8 x 6; <= 128: 16 x 8; <= 256: 32 x 8; wider: any), and
+  // a wide problem does not set the shared memory (and so the occupancy) of many
+  // narrow ones.  B is n x k with k <= n: n columns bound what a problem keeps in
+  // shared memory; beyond the cap it keeps what k columns it finds to fit, or
+  // works in its global buffer.
   const int tcb = prec == P32 ? 4 : 8;
   prof_batch_tag() = (long)v.size();
   const int kk = prec == P32 ? KK_SVD32 : KK_SVD64;
   cudaEvent_t pe = profiler().begin(kk, st.stream);
-  const int wcls[4] = {16, 48, 128, 1024};
-  std::vector<SvdRtDesc> part[4];
-  int nmx[4] = {1, 1, 1, 1};
+  static constexpr int wcls[5] = {16, 48, 128, 256, 1024}, grp[5] = {4, 8, 16, 32, 32};
+  std::vector<SvdRtDesc> part[5];
+  int nmx[5] = {1, 1, 1, 1, 1};
   for (auto& x : v) {
     int c = 0;
-    while (c < 3 && x.n > wcls[c]) ++c;
+    while (x.n > wcls[c]) ++c;
     part[c].push_back(x);
     nmx[c] = std::max(nmx[c], x.n);
   }
-  (void)nmax;
-  const SvdRtDesc* d[4] = {};
-  for (int c = 0; c < 4; ++c)
+  const SvdRtDesc* d[5] = {};
+  for (int c = 0; c < 5; ++c)
     if (!part[c].empty()) d[c] = st.push(part[c]);
   ForkJoin fj(st.stream);
   int li = 0;
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 4; c >= 0; --c) {  // the longest first
     if (part[c].empty()) continue;
-    const int smem = (int)std::min<size_t>(smem_cap, ((size_t)nmx[c] * nmx[c] * tcb + 15) & ~(size_t)15);
+    const size_t tail = svd_tail_bytes(nmx[c], tcb);
+    const int slot = (int)std::min<size_t>(
+        smem_cap, ((size_t)svd_ld(nmx[c], grp[c]) * nmx[c] * tcb + tail + 15) & ~(size_t)15);
     const unsigned g = (unsigned)part[c].size();
-    // one warp per column pair of the widest problem, up to 16 warps; up to 32
-    // when the class has fewer problems than SMs (nothing else to hide latency)
-    const int threads = std::min(g < 152 ? 1024 : 512, std::max(64, 32 * ((nmx[c] + 1) / 2)));
-    cudaStream_t s = fj.stream(li++);
+    // lanes for every pair of a problem that keeps all (class 1) or about half
+    // (wider) of its columns; more warps than that only wait at the rounds' barriers
+    const int pairs = c == 1 ? (nmx[c] + 1) / 2 : (nmx[c] + 3) / 4;
+    const int threads = std::min(g < 152 ? 1024 : 512, std::max(64, (pairs * grp[c] + 31) / 32 * 32));
     if (prec == P32)
-      k_svd_rt<float><<<g, threads, smem, s>>>(d[c], (int)g, 60, smem);
+      svd_rt_launch<float>(c, d[c], g, threads, slot, fj.stream(li++));
     else
-      k_svd_rt<double><<<g, threads, smem, s>>>(d[c], (int)g, 60, smem);
-    check_launch("k_svd_rt");
+      svd_rt_launch<double>(c, d[c], g, threads, slot, fj.stream(li++));
   }
   fj.join();
   profiler().end(kk, st.stream, pe);
