@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "descs.h"
+#include "devmath.cuh"
 #include "fp64_ops.cuh"
 
 namespace ifmm {
@@ -61,75 +62,6 @@ __global__ void k_copy_small(const CopyDesc* __restrict__ d, int nd) {
     double* o = D.dst + i + (long)j * D.ldd;
     *o = mode == 0 ? v : (mode == 1 ? *o + v : ((D.beta == 0.0) ? D.alpha * v : D.alpha * v + D.beta * (*o)));
   }
-}
-
-// ---------------------------------------------------------------- FP64 <-> FP32 on the integer pipes
-// GB300 executes double arithmetic and double<->float conversions on its narrow
-// FP64 pipe (about 2 operations per clock per SM).  The FP32 kernels read and
-// write FP64 storage, so they convert with integer operations on the IEEE-754
-// fields instead, folding an optional power-of-two scale 2^sh into the
-// exponent.  No path of either function uses a floating-point instruction (the
-// compiler would evaluate a rare-path hardware conversion on every call and
-// select).  d2f_pow2 rounds to nearest with ties away from zero (IEEE binary64
-// -> binary32 keeps the top 23 of 52 fraction bits; the first dropped bit
-// decides); results below the binary32 normal range become signed zero, above
-// it infinity; infinity and NaN stay infinity and (quiet) NaN.  f2d_pow2 widens
-// exactly (binary32 subnormals included); results below the binary64 normal
-// range become signed zero, above it infinity.
-__device__ __forceinline__ float d2f_pow2(double d, int sh) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned ah = hi & 0x7fffffffu, sg = hi & 0x80000000u;
-  if (ah >= 0x7ff00000u) {
-    const bool nan = ah > 0x7ff00000u || lo != 0u;
-    return __uint_as_float(sg | 0x7f800000u | (nan ? 0x400000u | ((ah & 0x000fffffu) << 3) : 0u));
-  }
-  const int e = (int)(ah >> 20) + sh;  // biased binary64 exponent after scaling
-  if (ah < 0x00100000u || e <= 896) return __uint_as_float(sg);
-  if (e >= 1151) return __uint_as_float(sg | 0x7f800000u);
-  unsigned f = ((unsigned)(e - 896) << 23) | ((ah & 0x000fffffu) << 3) | (lo >> 29);
-  f += (lo >> 28) & 1u;  // a carry into the exponent is the correct rounding
-  return __uint_as_float(sg | f);
-}
-__device__ __forceinline__ double f2d_pow2(float f, int sh) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned a = u & 0x7fffffffu, sg = u & 0x80000000u;
-  if (a == 0) return __hiloint2double((int)sg, 0);
-  if (a >= 0x7f800000u) {
-    const unsigned m = a & 0x007fffffu;  // NaN payload (0: infinity)
-    return __hiloint2double((int)(sg | 0x7ff00000u | (m ? 0x80000u | (m >> 3) : 0u)), (int)(m << 29));
-  }
-  unsigned mant;
-  int e;  // biased binary64 exponent
-  if (a < 0x00800000u) {  // subnormal: a 2^-149, normalised
-    const int lz = __clz((int)a) - 8;
-    mant = (a << lz) & 0x007fffffu;
-    e = 897 - lz + sh;
-  } else {
-    mant = a & 0x007fffffu;
-    e = (int)(a >> 23) + 896 + sh;
-  }
-  if (e <= 0) return __hiloint2double((int)sg, 0);
-  if (e >= 2047) return __hiloint2double((int)(sg | 0x7ff00000u), 0);
-  return __hiloint2double((int)(sg | ((unsigned)e << 20) | (mant >> 3)), (int)(mant << 29));
-}
-// biased binary64 exponent of |d| (0 for zero and subnormals, 2047 for inf/NaN)
-__device__ __forceinline__ int dexp(double d) { return (int)(((unsigned)__double2hiint(d) & 0x7fffffffu) >> 20); }
-
-// value of a double as the arithmetic type TC, times 2^sh
-template <typename TC>
-__device__ __forceinline__ TC ld_tc(double d, int sh = 0) {
-  if constexpr (sizeof(TC) == 4)
-    return d2f_pow2(d, sh);
-  else
-    return sh ? ldexp(d, sh) : d;
-}
-// a TC value times 2^sh, as a double
-template <typename TC>
-__device__ __forceinline__ double st_tc(TC v, int sh = 0) {
-  if constexpr (sizeof(TC) == 4)
-    return f2d_pow2(v, sh);
-  else
-    return sh ? ldexp(v, sh) : v;
 }
 
 // RB: the operands are rounded to bfloat16 before the (FP32) multiply-add.
@@ -508,12 +440,6 @@ __global__ void __launch_bounds__(256, 2) k_gemm_tc(const GemmDesc* __restrict__
 }
 
 // ---------------------------------------------------------------- reductions
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // block-wide sum; scratch holds >= 32 doubles; every thread gets the result
 __device__ double block_sum(double v, double* scratch) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -551,18 +477,6 @@ __host__ __device__ __forceinline__ size_t inv_slot_bytes(int n, int R) {
   const size_t nc = ((size_t)n + R - 1) / R;
   return ((size_t)n * nc + 3 * (size_t)n + nc) * sizeof(double) + ((sizeof(int) * (size_t)n + 15) & ~(size_t)15);
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
-// the warp's largest key (hi, lo), lexicographic, and the smallest index among
-// the lanes that hold it; every lane gets the result
-__device__ __forceinline__ void warp_max_key(unsigned& hi, unsigned& lo, int& i) {
-  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-  i = (int)__reduce_min_sync(0xffffffffu, (hi == mh && lo == ml) ? (unsigned)i : 0x7fffffffu);
-  hi = mh;
-  lo = ml;
-}
-
 // V: rows per thread, n <= V * blockDim.x
 template <int V>
 __global__ void __launch_bounds__(512) k_inv(const InvDesc* __restrict__ d, int nd) {
@@ -838,13 +752,6 @@ __global__ void k_gjb_colswap(const InvDesc* __restrict__ d, int nd, const doubl
 // One CTA per matrix.  Column k: v = x - alpha e1 with alpha = -sign(x_0)||x||,
 // H = I - 2 v v^T / (v^T v) applied to the trailing columns (one warp per column).
 // Storage is double; TC is the arithmetic type of the dot products and updates.
-template <typename TC>
-__device__ __forceinline__ TC warp_sum_t(TC v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Apply H = I - t v v^T (v_0 = 1, v_i = x_i for i >= 1) to the trailing
 // columns k+1..n-1 of A (rows k..k+len-1).  Each column's dot product and
 // update is split into S row segments when there are fewer trailing columns
@@ -1070,720 +977,6 @@ __global__ void k_qrcp(const QrcpDesc* __restrict__ d, int nd) {
   if (threadIdx.x == 0) {
     D.kout[0] = k;
     if (D.tail) D.tail[0] = (k < kmax && s_capped) ? s_tailv : 0.0;
-  }
-}
-
-// ---------------------------------------------------------------- Householder QR in shared memory
-// The factorisations of k_qr (PIV = false) and k_qrcp (PIV = true) for blocks
-// that fit in shared memory in the arithmetic type TC: the block is read from
-// global memory once, factorised in shared memory, and written back once.
-// On the way in it is multiplied by a power of two (exact) that brings its
-// largest magnitude into [0.5, 1): squared column norms of FP32 blocks whose
-// entries are ~1e-12 would otherwise fall out of the FP32 normal range.  R is
-// scaled back (exactly) on the way out.  The Householder vector of step k,
-// v_0 = 1, v_i = sc x_i, is formed on the fly from the untouched column and
-// never stored; the column is zeroed below the diagonal on write-back.  The
-// norm of every pivot candidate is downdated right after its column has been
-// updated, in the same pass.
-// Slot of one problem: A (m x n, ld m) | nrm (n) | ref (n), in TC | jp (n ints).
-__host__ __device__ __forceinline__ size_t qr_slot_bytes(int m, int n, int tc_bytes) {
-  return (((size_t)m * n + 2 * (size_t)n) * tc_bytes + sizeof(int) * (size_t)n + 15) & ~(size_t)15;
-}
-
-// exponent shift that brings a block whose largest |entry| has biased binary64
-// exponent emax into [0.5, 1) (0 for an all-zero block or one with inf/NaN)
-__device__ __forceinline__ int pow2_shift(int emax) { return (emax <= 0 || emax >= 2047) ? 0 : 1022 - emax; }
-
-// Applies H = I - tau v v^T (v_0 = 1, v_i = sc x_i) to the cnt <= G columns
-// j0.. of the trailing block (rows k..k+len-1, ld m) with one warp: G independent
-// dot products per row sweep and G interleaved butterfly reductions, so the
-// shared-memory and shuffle latencies of the columns overlap.
-template <typename TC, int G>
-__device__ __forceinline__ void reflect_group(TC* A, int m, int k, int len, const TC* x, TC sc, TC tau, int j0,
-                                              int cnt, int lane) {
-  TC* y[G];
-#pragma unroll
-  for (int u = 0; u < G; ++u) y[u] = A + k + (size_t)(j0 + (u < cnt ? u : cnt - 1)) * m;
-  TC acc[G];
-#pragma unroll
-  for (int u = 0; u < G; ++u) acc[u] = 0;
-  for (int i = lane; i < len; i += 32) {
-    const TC vi = (i == 0) ? (TC)1 : sc * x[i];
-#pragma unroll
-    for (int u = 0; u < G; ++u) acc[u] += vi * y[u][i];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int u = 0; u < G; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
-  for (int i = lane; i < len; i += 32) {
-    const TC vi = (i == 0) ? (TC)1 : sc * x[i];
-#pragma unroll
-    for (int u = 0; u < G; ++u)
-      if (u < cnt) y[u][i] -= (acc[u] * tau) * vi;
-  }
-}
-
-// (row, column) of the flat column-major index e = i + j m, advanced by a fixed
-// stride without a division per step
-struct FlatIdx {
-  int i, j, di, dj, m;
-  __device__ __forceinline__ FlatIdx(int e0, int stride, int m_) : m(m_ > 0 ? m_ : 1) {
-    i = e0 % m;
-    j = e0 / m;
-    di = stride % m;
-    dj = stride / m;
-  }
-  __device__ __forceinline__ void next() {
-    i += di;
-    j += dj;
-    if (i >= m) {
-      i -= m;
-      ++j;
-    }
-  }
-};
-
-// physical row of logical row i (QrcpDesc::rb, rs)
-__device__ __forceinline__ long qr_row(const QrcpDesc& D, int i) {
-  return D.rb > 0 ? (long)(i / D.rb) * D.rs + i % D.rb : (long)i;
-}
-
-// One warp per problem; blockDim.x / 32 problems per CTA; slot_bytes of
-// dynamic shared memory per warp.  Only __syncwarp is used.
-template <typename TC, bool PIV>
-__global__ void k_qr_warp(const QrcpDesc* __restrict__ d, int nd, int slot_bytes) {
-  extern __shared__ __align__(16) unsigned char qsm[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int di = blockIdx.x * (blockDim.x >> 5) + w;
-  if (di >= nd) return;
-  const QrcpDesc D = d[di];
-  const int m = D.m, n = D.n;
-  const long ld = D.ld;
-  const int mn = m * n;
-  TC* A = (TC*)(qsm + (size_t)w * slot_bytes);
-  TC* nrm = A + mn;
-  TC* ref = nrm + n;
-  int* jp = (int*)(ref + n);
-  int em = 0;
-  {
-    FlatIdx x(lane, 32, m);
-    for (int e = lane; e < mn; e += 32, x.next()) em = max(em, dexp(D.A[qr_row(D, x.i) + (long)x.j * ld]));
-  }
-  const int sh = pow2_shift((int)__reduce_max_sync(0xffffffffu, (unsigned)em));
-  {
-    FlatIdx x(lane, 32, m);
-    for (int e = lane; e < mn; e += 32, x.next()) A[e] = ld_tc<TC>(D.A[qr_row(D, x.i) + (long)x.j * ld], sh);
-  }
-  __syncwarp();
-  if (PIV) {
-    for (int j = 0; j < n; ++j) {
-      const TC* c = A + (size_t)j * m;
-      TC ss = 0;
-      for (int i = lane; i < m; i += 32) ss += c[i] * c[i];
-      ss = warp_sum_t<TC>(ss);
-      if (lane == 0) {
-        nrm[j] = ss;
-        ref[j] = ss;
-        jp[j] = j;
-      }
-    }
-    __syncwarp();
-  }
-  const int kmax = m < n ? m : n;
-  TC tau2 = 0, first = 0;
-  double tailv = 0.0;
-  bool capped = false;
-  int k = 0;
-  for (; k < kmax; ++k) {
-    if (PIV) {
-      TC best = -1;
-      int bi = n;
-      for (int j = k + lane; j < n; j += 32) {
-        const TC v = nrm[j];
-        if (v > best || (v == best && j < bi)) { best = v; bi = j; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const TC ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-      }
-      if (k == 0) {
-        tau2 = (TC)(D.tau_rel * D.tau_rel) * best;
-        first = best;
-      }
-      bool stop = !(best > tau2) || !(best > (TC)0) || bi >= n;
-      if (!stop && D.kcap > 0 && k >= D.kcap) {
-        stop = true;
-        capped = true;
-        tailv = (first > (TC)0) ? sqrt((double)best / (double)first) : 0.0;
-      }
-      if (stop) break;
-      if (bi != k) {
-        TC* ck = A + (size_t)k * m;
-        TC* cp = A + (size_t)bi * m;
-        for (int i = lane; i < m; i += 32) {
-          const TC t = ck[i];
-          ck[i] = cp[i];
-          cp[i] = t;
-        }
-        if (lane == 0) {
-          TC t = nrm[k]; nrm[k] = nrm[bi]; nrm[bi] = t;
-          t = ref[k]; ref[k] = ref[bi]; ref[bi] = t;
-          const int q = jp[k]; jp[k] = jp[bi]; jp[bi] = q;
-        }
-        __syncwarp();
-      }
-    }
-    TC* x = A + k + (size_t)k * m;
-    const int len = m - k;
-    TC ss = 0;
-    for (int i = lane; i < len; i += 32)
-      if (i > 0) ss += x[i] * x[i];
-    ss = warp_sum_t<TC>(ss);
-    const TC x0 = x[0];
-    const TC nr = sqrt(x0 * x0 + ss);
-    TC alpha = x0, tau = 0, sc = 0;
-    if (!(nr == (TC)0 || ss == (TC)0)) {
-      alpha = (x0 >= (TC)0) ? -nr : nr;
-      tau = (alpha - x0) / alpha;
-      sc = (TC)1 / (x0 - alpha);
-    }
-    for (int j0 = k + 1; j0 < n; j0 += 4) {
-      const int cnt = min(4, n - j0);
-      if (tau != (TC)0) reflect_group<TC, 4>(A, m, k, len, x, sc, tau, j0, cnt, lane);
-      if (PIV) {
-        for (int u = 0; u < cnt; ++u) {
-          const int j = j0 + u;
-          const TC* y = A + k + (size_t)j * m;
-          const TC nj = nrm[j], rj = ref[j];
-          const TC r = __shfl_sync(0xffffffffu, lane == 0 ? y[0] : (TC)0, 0);
-          TC nv = nj - r * r;
-          if (!(nv > (TC)1e-2 * rj)) {  // two digits lost: recompute from the column
-            TC s2 = 0;
-            for (int i = lane; i < len; i += 32)
-              if (i > 0) s2 += y[i] * y[i];
-            nv = warp_sum_t<TC>(s2);
-            if (lane == 0) ref[j] = nv;
-          }
-          if (lane == 0) nrm[j] = nv;
-        }
-      }
-    }
-    if (lane == 0) x[0] = alpha;
-    __syncwarp();
-  }
-  {
-    FlatIdx x(lane, 32, m);
-    for (int e = lane; e < mn; e += 32, x.next()) {
-      const TC v = (x.j < k && x.i > x.j) ? (TC)0 : A[e];
-      D.A[qr_row(D, x.i) + (long)x.j * ld] = st_tc<TC>(v, -sh);
-    }
-  }
-  if (PIV) {
-    for (int j = lane; j < n; j += 32) D.jpvt[j] = jp[j];
-    if (lane == 0) {
-      D.kout[0] = k;
-      if (D.tail) D.tail[0] = (k < kmax && capped) ? tailv : 0.0;
-    }
-  }
-}
-
-// One CTA (<= 1024 threads) per problem, the block in dynamic shared memory.
-// Per column step: one barrier for the pivot search, one after a column swap,
-// one for the reflector norm, one between the segment dot products and the
-// update, and one closing the step (plus one more in the rare step where a
-// downdated norm has to be recomputed).
-template <typename TC, bool PIV>
-__global__ void __launch_bounds__(1024) k_qr_cta(const QrcpDesc* __restrict__ d, int nd) {
-  if ((int)blockIdx.x >= nd) return;
-  const QrcpDesc D = d[blockIdx.x];
-  const int m = D.m, n = D.n;
-  const long ld = D.ld;
-  const int mn = m * n;
-  extern __shared__ __align__(16) unsigned char qsm[];
-  TC* A = (TC*)qsm;
-  TC* nrm = A + mn;
-  TC* ref = nrm + n;
-  int* jp = (int*)(ref + n);
-  __shared__ TC part[32];
-  __shared__ unsigned char flag[1024];
-  __shared__ TC red_s[32], red_v[32];
-  __shared__ int red_i[32];
-  const int tid = threadIdx.x, nt_ = blockDim.x;
-  const int lane = tid & 31, w = tid >> 5, nw = nt_ >> 5;
-  int em = 0;
-  {
-    FlatIdx x(tid, nt_, m);
-    for (int e = tid; e < mn; e += nt_, x.next()) em = max(em, dexp(D.A[qr_row(D, x.i) + (long)x.j * ld]));
-  }
-  em = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
-  if (lane == 0) red_i[w] = em;
-  __syncthreads();
-  em = 0;
-  for (int i = 0; i < nw; ++i) em = max(em, red_i[i]);
-  const int sh = pow2_shift(em);
-  {
-    FlatIdx x(tid, nt_, m);
-    for (int e = tid; e < mn; e += nt_, x.next()) A[e] = ld_tc<TC>(D.A[qr_row(D, x.i) + (long)x.j * ld], sh);
-  }
-  for (int j = tid; j < n; j += nt_) flag[j] = 0;
-  __syncthreads();
-  if (PIV) {
-    for (int j = w; j < n; j += nw) {
-      const TC* c = A + (size_t)j * m;
-      TC ss = 0;
-      for (int i = lane; i < m; i += 32) ss += c[i] * c[i];
-      ss = warp_sum_t<TC>(ss);
-      if (lane == 0) {
-        nrm[j] = ss;
-        ref[j] = ss;
-        jp[j] = j;
-      }
-    }
-    __syncthreads();
-  }
-  const int kmax = m < n ? m : n;
-  TC tau2 = 0, first = 0;
-  double tailv = 0.0;
-  bool capped = false;
-  int k = 0;
-  for (; k < kmax; ++k) {
-    if (PIV) {
-      TC best = -1;
-      int bi = n;
-      for (int j = k + tid; j < n; j += nt_) {
-        const TC v = nrm[j];
-        if (v > best || (v == best && j < bi)) { best = v; bi = j; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const TC ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-      }
-      if (lane == 0) {
-        red_v[w] = best;
-        red_i[w] = bi;
-      }
-      __syncthreads();
-      best = -1;
-      bi = n;
-      for (int i = 0; i < nw; ++i)
-        if (red_v[i] > best || (red_v[i] == best && red_i[i] < bi)) { best = red_v[i]; bi = red_i[i]; }
-      if (k == 0) {
-        tau2 = (TC)(D.tau_rel * D.tau_rel) * best;
-        first = best;
-      }
-      bool stop = !(best > tau2) || !(best > (TC)0) || bi >= n;
-      if (!stop && D.kcap > 0 && k >= D.kcap) {
-        stop = true;
-        capped = true;
-        tailv = (first > (TC)0) ? sqrt((double)best / (double)first) : 0.0;
-      }
-      if (stop) break;
-      if (bi != k) {
-        TC* ck = A + (size_t)k * m;
-        TC* cp = A + (size_t)bi * m;
-        for (int i = tid; i < m; i += nt_) {
-          const TC t = ck[i];
-          ck[i] = cp[i];
-          cp[i] = t;
-        }
-        if (tid == 0) {
-          TC t = nrm[k]; nrm[k] = nrm[bi]; nrm[bi] = t;
-          t = ref[k]; ref[k] = ref[bi]; ref[bi] = t;
-          const int q = jp[k]; jp[k] = jp[bi]; jp[bi] = q;
-        }
-        __syncthreads();
-      }
-    }
-    TC* x = A + k + (size_t)k * m;
-    const int len = m - k;
-    TC ss = 0;
-    for (int i = tid; i < len; i += nt_)
-      if (i > 0) ss += x[i] * x[i];
-    ss = warp_sum_t<TC>(ss);
-    if (lane == 0) red_s[w] = ss;
-    __syncthreads();
-    ss = 0;
-    for (int i = 0; i < nw; ++i) ss += red_s[i];
-    const TC x0 = x[0];
-    const TC nr = sqrt(x0 * x0 + ss);
-    TC alpha = x0, tau = 0, sc = 0;
-    if (!(nr == (TC)0 || ss == (TC)0)) {
-      alpha = (x0 >= (TC)0) ? -nr : nr;
-      tau = (alpha - x0) / alpha;
-      sc = (TC)1 / (x0 - alpha);
-    }
-    const int ntr = n - k - 1;
-    int need = 0;
-    if (ntr > 0 && tau != (TC)0) {
-      // a trailing column is split into S row segments when there are fewer
-      // columns than warps (then ntr * S <= nw); segment sums are added in a
-      // fixed order
-      int S = nw / ntr;
-      const int smax = (len + 63) / 64;
-      if (S > smax) S = smax;
-      if (S < 1) S = 1;
-      if (S == 1) {
-        // groups of G consecutive columns, round-robin over the warps
-        const int G = ntr >= 4 * nw ? 4 : (ntr >= 2 * nw ? 2 : 1);
-        const int ng = (ntr + G - 1) / G;
-        for (int g = w; g < ng; g += nw) {
-          const int j0 = k + 1 + g * G;
-          const int cnt = min(G, n - j0);
-          if (G == 4)
-            reflect_group<TC, 4>(A, m, k, len, x, sc, tau, j0, cnt, lane);
-          else if (G == 2)
-            reflect_group<TC, 2>(A, m, k, len, x, sc, tau, j0, cnt, lane);
-          else
-            reflect_group<TC, 1>(A, m, k, len, x, sc, tau, j0, cnt, lane);
-          if (PIV && lane == 0) {
-            for (int u = 0; u < cnt; ++u) {
-              const int j = j0 + u;
-              const TC r = A[k + (size_t)j * m];
-              const TC nv = nrm[j] - r * r;
-              nrm[j] = nv;
-              if (!(nv > (TC)1e-2 * ref[j])) {
-                flag[j] = 1;
-                need = 1;
-              }
-            }
-          }
-        }
-      } else {
-        const int seg = (len + S - 1) / S;
-        const int items = ntr * S;
-        for (int it = w; it < items; it += nw) {
-          const int jj = it / S, sg = it % S;
-          const TC* y = A + k + (size_t)(k + 1 + jj) * m;
-          const int r0 = sg * seg, r1 = min(len, r0 + seg);
-          TC dot = 0;
-          for (int i = r0 + lane; i < r1; i += 32) dot += (i == 0 ? (TC)1 : sc * x[i]) * y[i];
-          dot = warp_sum_t<TC>(dot);
-          if (lane == 0) part[it] = dot;
-        }
-        __syncthreads();
-        for (int it = w; it < items; it += nw) {
-          const int jj = it / S, sg = it % S;
-          const int j = k + 1 + jj;
-          TC* y = A + k + (size_t)j * m;
-          TC dot = 0;
-          for (int q = 0; q < S; ++q) dot += part[jj * S + q];
-          dot *= tau;
-          const int r0 = sg * seg, r1 = min(len, r0 + seg);
-          for (int i = r0 + lane; i < r1; i += 32) y[i] -= dot * (i == 0 ? (TC)1 : sc * x[i]);
-          if (PIV && sg == 0 && lane == 0) {
-            const TC r = y[0];
-            const TC nv = nrm[j] - r * r;
-            nrm[j] = nv;
-            if (!(nv > (TC)1e-2 * ref[j])) {
-              flag[j] = 1;
-              need = 1;
-            }
-          }
-        }
-      }
-    } else if (PIV && ntr > 0) {
-      for (int j = k + 1 + tid; j < n; j += nt_) {
-        const TC r = A[k + (size_t)j * m];
-        const TC nv = nrm[j] - r * r;
-        nrm[j] = nv;
-        if (!(nv > (TC)1e-2 * ref[j])) {
-          flag[j] = 1;
-          need = 1;
-        }
-      }
-    }
-    const int any = __syncthreads_or(need);
-    if (PIV && any) {  // two digits lost: recompute those norms from the columns
-      for (int j = k + 1 + w; j < n; j += nw) {
-        if (!flag[j]) continue;
-        const TC* y = A + k + (size_t)j * m;
-        TC s2 = 0;
-        for (int i = lane; i < len; i += 32)
-          if (i > 0) s2 += y[i] * y[i];
-        s2 = warp_sum_t<TC>(s2);
-        if (lane == 0) {
-          nrm[j] = s2;
-          ref[j] = s2;
-          flag[j] = 0;
-        }
-      }
-      __syncthreads();
-    }
-    if (tid == 0) x[0] = alpha;
-  }
-  __syncthreads();
-  {
-    FlatIdx x(tid, nt_, m);
-    for (int e = tid; e < mn; e += nt_, x.next()) {
-      const TC v = (x.j < k && x.i > x.j) ? (TC)0 : A[e];
-      D.A[qr_row(D, x.i) + (long)x.j * ld] = st_tc<TC>(v, -sh);
-    }
-  }
-  if (PIV) {
-    for (int j = tid; j < n; j += nt_) D.jpvt[j] = jp[j];
-    if (tid == 0) {
-      D.kout[0] = k;
-      if (D.tail) D.tail[0] = (k < kmax && capped) ? tailv : 0.0;
-    }
-  }
-}
-
-// ---------------------------------------------------------------- Householder QR across a cluster
-// The same factorisations as k_qr_cta for blocks too large for one CTA's shared
-// memory: the rows are split over the R CTAs of a thread-block cluster (CTA r
-// holds logical rows [r*chunk, (r+1)*chunk) of all n columns, chunk = ceil(m/R)),
-// and the CTAs exchange through distributed shared memory.  Every CTA keeps the
-// column norms, the pivot order and the reflector scalars replicated, computed by
-// the same operations in the same order, so every decision (pivot, stop, norm
-// recompute) is identical cluster-wide.  Per column step there are two cluster
-// barriers: after the partial reflector norms (plus the diagonal entry from the
-// CTA that owns row k), and after the partial dot products (plus the owner's row k,
-// from which every CTA forms row k of R for the norm downdate).  The exchange
-// buffers alternate between even and odd steps, so a buffer is rewritten only
-// after every CTA has passed the barrier that follows its last read.
-// Slot: A (chunk x n, ld chunk) | nrm, ref (n) | xd (2n) | xr (2n) | xs (8), in TC | jp (n ints).
-__host__ __device__ __forceinline__ size_t qr_cluster_slot_bytes(int m, int n, int R, int tc_bytes) {
-  const size_t chunk = ((size_t)m + R - 1) / R;
-  return ((chunk * n + 6 * (size_t)n + 8) * tc_bytes + sizeof(int) * (size_t)n + 15) & ~(size_t)15;
-}
-
-template <typename TC, bool PIV>
-__global__ void __launch_bounds__(512) k_qr_cluster(const QrcpDesc* __restrict__ d, int nd) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int R = (int)cl.num_blocks();
-  const int rank = (int)cl.block_rank();
-  const int pi = (int)(blockIdx.x / R);
-  const QrcpDesc D = d[pi < nd ? pi : nd - 1];
-  const int m = D.m, n = D.n;
-  const long ld = D.ld;
-  const int chunk = (m + R - 1) / R;
-  const int r0 = min(m, rank * chunk), ml = min(m, r0 + chunk) - r0;
-  const int mlp = chunk > 0 ? chunk : 1;
-  extern __shared__ __align__(16) unsigned char qsm[];
-  TC* A = (TC*)qsm;
-  TC* nrm = A + (size_t)mlp * n;
-  TC* ref = nrm + n;
-  TC* xd = ref + n;
-  TC* xr = xd + 2 * n;
-  TC* xs = xr + 2 * n;
-  int* jp = (int*)(xs + 8);
-  __shared__ unsigned char flag[1024];
-  __shared__ TC red_s[32], red_v[32];
-  __shared__ int red_i[32];
-  __shared__ int xg;
-  const int tid = threadIdx.x, nt_ = blockDim.x;
-  const int lane = tid & 31, w = tid >> 5, nw = nt_ >> 5;
-  // power-of-two scale from the cluster-wide largest magnitude
-  int em = 0;
-  for (int e = tid; e < ml * n; e += nt_) em = max(em, dexp(D.A[(r0 + e % ml) + (long)(e / ml) * ld]));
-  em = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
-  if (lane == 0) red_i[w] = em;
-  __syncthreads();
-  if (tid == 0) {
-    int g = 0;
-    for (int i = 0; i < nw; ++i) g = max(g, red_i[i]);
-    xg = g;
-  }
-  for (int j = tid; j < n; j += nt_) flag[j] = 0;
-  cl.sync();
-  em = 0;
-  for (int r = 0; r < R; ++r) em = max(em, *cl.map_shared_rank(&xg, r));
-  const int sh = pow2_shift(em);
-  for (int e = tid; e < ml * n; e += nt_) {
-    const int li = e % ml, j = e / ml;
-    A[li + (size_t)j * mlp] = ld_tc<TC>(D.A[(r0 + li) + (long)j * ld], sh);
-  }
-  __syncthreads();
-  if (PIV) {
-    for (int j = w; j < n; j += nw) {
-      const TC* c = A + (size_t)j * mlp;
-      TC ss = 0;
-      for (int i = lane; i < ml; i += 32) ss += c[i] * c[i];
-      ss = warp_sum_t<TC>(ss);
-      if (lane == 0) xd[j] = ss;
-    }
-    cl.sync();
-    for (int j = tid; j < n; j += nt_) {
-      TC s = 0;
-      for (int r = 0; r < R; ++r) s += cl.map_shared_rank(xd, r)[j];
-      nrm[j] = s;
-      ref[j] = s;
-      jp[j] = j;
-    }
-    __syncthreads();
-  }
-  const int kmax = m < n ? m : n;
-  TC tau2 = 0, first = 0;
-  double tailv = 0.0;
-  bool capped = false;
-  int k = 0;
-  for (; k < kmax; ++k) {
-    const int buf = k & 1;
-    if (PIV) {
-      TC best = -1;
-      int bi = n;
-      for (int j = k + tid; j < n; j += nt_) {
-        const TC v = nrm[j];
-        if (v > best || (v == best && j < bi)) { best = v; bi = j; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const TC ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-      }
-      if (lane == 0) {
-        red_v[w] = best;
-        red_i[w] = bi;
-      }
-      __syncthreads();
-      best = -1;
-      bi = n;
-      for (int i = 0; i < nw; ++i)
-        if (red_v[i] > best || (red_v[i] == best && red_i[i] < bi)) { best = red_v[i]; bi = red_i[i]; }
-      if (k == 0) {
-        tau2 = (TC)(D.tau_rel * D.tau_rel) * best;
-        first = best;
-      }
-      bool stop = !(best > tau2) || !(best > (TC)0) || bi >= n;
-      if (!stop && D.kcap > 0 && k >= D.kcap) {
-        stop = true;
-        capped = true;
-        tailv = (first > (TC)0) ? sqrt((double)best / (double)first) : 0.0;
-      }
-      if (stop) break;
-      if (bi != k) {
-        TC* ck = A + (size_t)k * mlp;
-        TC* cp = A + (size_t)bi * mlp;
-        for (int i = tid; i < ml; i += nt_) {
-          const TC t = ck[i];
-          ck[i] = cp[i];
-          cp[i] = t;
-        }
-        if (tid == 0) {
-          TC t = nrm[k]; nrm[k] = nrm[bi]; nrm[bi] = t;
-          t = ref[k]; ref[k] = ref[bi]; ref[bi] = t;
-          const int q = jp[k]; jp[k] = jp[bi]; jp[bi] = q;
-        }
-        __syncthreads();
-      }
-    }
-    const int owner = k / chunk;
-    const int lk = k - r0;  // local row of k (in [0, ml) on the owner)
-    // local rows li >= l0 hold logical rows >= k
-    const int l0 = max(0, k - r0);
-    const TC* xk = A + (size_t)k * mlp;
-    TC ss = 0;
-    for (int li = l0 + tid; li < ml; li += nt_)
-      if (r0 + li > k) ss += xk[li] * xk[li];
-    ss = warp_sum_t<TC>(ss);
-    if (lane == 0) red_s[w] = ss;
-    __syncthreads();
-    if (tid == 0) {
-      TC s = 0;
-      for (int i = 0; i < nw; ++i) s += red_s[i];
-      xs[4 * buf] = s;
-      if (rank == owner) xs[4 * buf + 1] = xk[lk];
-    }
-    cl.sync();
-    ss = 0;
-    for (int r = 0; r < R; ++r) ss += cl.map_shared_rank(xs, r)[4 * buf];
-    const TC x0 = cl.map_shared_rank(xs, owner)[4 * buf + 1];
-    const TC nr = sqrt(x0 * x0 + ss);
-    TC alpha = x0, tau = 0, sc = 0;
-    if (!(nr == (TC)0 || ss == (TC)0)) {
-      alpha = (x0 >= (TC)0) ? -nr : nr;
-      tau = (alpha - x0) / alpha;
-      sc = (TC)1 / (x0 - alpha);
-    }
-    const int ntr = n - k - 1;
-    TC* xdb = xd + (size_t)buf * n;
-    TC* xrb = xr + (size_t)buf * n;
-    if (ntr > 0 && tau != (TC)0) {
-      for (int j = k + 1 + w; j < n; j += nw) {
-        const TC* y = A + (size_t)j * mlp;
-        TC acc = 0;
-        for (int li = l0 + lane; li < ml; li += 32) {
-          const TC vi = (r0 + li == k) ? (TC)1 : sc * xk[li];
-          acc += vi * y[li];
-        }
-        acc = warp_sum_t<TC>(acc);
-        if (lane == 0) xdb[j] = acc;
-      }
-    }
-    if (rank == owner)
-      for (int j = k + 1 + tid; j < n; j += nt_) xrb[j] = A[lk + (size_t)j * mlp];
-    cl.sync();
-    int need = 0;
-    if (ntr > 0) {
-      const TC* xro = cl.map_shared_rank(xrb, owner);
-      for (int j = k + 1 + w; j < n; j += nw) {
-        TC dj = 0;
-        if (tau != (TC)0) {
-          for (int r = 0; r < R; ++r) dj += cl.map_shared_rank(xdb, r)[j];
-          dj *= tau;
-          TC* y = A + (size_t)j * mlp;
-          for (int li = l0 + lane; li < ml; li += 32) {
-            const TC vi = (r0 + li == k) ? (TC)1 : sc * xk[li];
-            y[li] -= dj * vi;
-          }
-        }
-        if (PIV && lane == 0) {
-          const TC rkj = xro[j] - dj;  // row k of R: the owner's row k minus d_j v_k, v_k = 1
-          const TC nv = nrm[j] - rkj * rkj;
-          nrm[j] = nv;
-          if (!(nv > (TC)1e-2 * ref[j])) {
-            flag[j] = 1;
-            need = 1;
-          }
-        }
-      }
-    }
-    const int any = __syncthreads_or(need);
-    if (PIV && any) {  // two digits lost (identically in every CTA): recompute
-      TC* xdo = xd + (size_t)(buf ^ 1) * n;
-      for (int j = k + 1 + w; j < n; j += nw) {
-        if (!flag[j]) continue;
-        const TC* y = A + (size_t)j * mlp;
-        TC s2 = 0;
-        for (int li = l0 + lane; li < ml; li += 32)
-          if (r0 + li > k) s2 += y[li] * y[li];
-        s2 = warp_sum_t<TC>(s2);
-        if (lane == 0) xdo[j] = s2;
-      }
-      cl.sync();
-      for (int j = k + 1 + tid; j < n; j += nt_) {
-        if (!flag[j]) continue;
-        TC s = 0;
-        for (int r = 0; r < R; ++r) s += cl.map_shared_rank(xdo, r)[j];
-        nrm[j] = s;
-        ref[j] = s;
-        flag[j] = 0;
-      }
-    }
-    if (rank == owner && tid == 0) A[lk + (size_t)k * mlp] = alpha;
-    __syncthreads();
-  }
-  // no CTA leaves while another may still read its shared memory
-  cl.sync();
-  for (int e = tid; e < ml * n; e += nt_) {
-    const int li = e % ml, j = e / ml;
-    const int i = r0 + li;
-    const TC v = (j < k && i > j) ? (TC)0 : A[li + (size_t)j * mlp];
-    D.A[i + (long)j * ld] = st_tc<TC>(v, -sh);
-  }
-  if (PIV && rank == 0) {
-    for (int j = tid; j < n; j += nt_) D.jpvt[j] = jp[j];
-    if (tid == 0) {
-      D.kout[0] = k;
-      if (D.tail) D.tail[0] = (k < kmax && capped) ? tailv : 0.0;
-    }
   }
 }
 

@@ -7,7 +7,7 @@
 
 namespace ifmm {
 
-__device__ __noinline__ double rsqrt_rare(double a) { return rsqrt(a); }
+static __device__ __noinline__ double rsqrt_rare(double a) { return rsqrt(a); }
 // 1/sqrt(a) to about an ulp: a = m 4^k, 1 <= m < 4; y0 = rsqrt(float(m)) 2^-k to
 // ~2^-22, then one step y0 (1 + e/2 + 3 e^2 / 8), e = 1 - a y0^2 (the next term is
 // below 2^-65).  Zero, subnormal, negative and non-finite arguments take CUDA's.

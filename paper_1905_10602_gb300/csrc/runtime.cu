@@ -11,6 +11,7 @@
 #include "matvec_fp64.cuh"
 #include "krylov.cuh"
 #include "ifmm_kernels.h"
+#include "qr.h"
 #include "runtime.h"
 
 namespace ifmm {
@@ -495,178 +496,167 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
   }
 }
 
-// Size buckets of the Householder QR launches.  A problem whose shared-memory
-// slot (block + norms, in the arithmetic type) is at most kQrWarpSlot bytes is
-// factorised by one warp; one of at most kQrCtaSmem bytes by one CTA with the
-// block in shared memory.  A taller block is first reduced in place: its rows
-// are cut into chunks that fit, each chunk is factorised (unpivoted), and the
-// stacked chunk R factors -- the same column space, column norms and R up to
-// signs -- are factorised as the logical matrix (rows addressed through
-// QrcpDesc::rb, rs), when they fit.  Anything else goes to the global-memory
-// kernels.
-static constexpr size_t kQrWarpSlot = 12 * 1024;
-static constexpr size_t kQrCtaSmem = 220 * 1024;
-// Shared memory a QR problem may use per CTA; IFMM_QR_CTA_LIMIT_KB (<= 220)
-// lowers it, which routes smaller problems through the tall reduction, the
-// cluster and the global-memory kernels (used by the tests of those paths).
+// How a QR problem is launched.  At most 16 columns and 128 rows: a warp per
+// problem.  Else the class by rows and a cluster of R CTAs with just the warps its
+// columns need (qr.cuh); R is what the registers require and, while the whole
+// launch leaves SMs idle, more (FP64: up to two CTAs per SM, its pipe being the
+// bound; FP32: one, where a split only adds the cluster barriers' latency).
+// Blocks taller than the largest class are first reduced in place: row chunks are
+// factorised (unpivoted) and the stacked chunk R factors -- the same column
+// space, column norms and R up to signs -- are factorised as the logical matrix
+// (rows addressed through QrcpDesc::rb, rs).  Anything else goes to the
+// global-memory kernels.
+static constexpr size_t kQrCtaBytes = 220 * 1024;
+// Bytes of a block that one CTA may hold; IFMM_QR_CTA_LIMIT_KB (<= 220) lowers it,
+// which spreads smaller problems over clusters (of at most 8 CTAs then), reduces
+// them by chunks or sends them to the global-memory kernels (used by the tests of
+// those paths).
 static size_t qr_cta_limit() {
   static const size_t lim = [] {
     const char* e = getenv("IFMM_QR_CTA_LIMIT_KB");
     const long kb = e ? atol(e) : 0;
-    return (kb >= 4 && kb <= 220) ? (size_t)kb * 1024 : kQrCtaSmem;
+    return (kb >= 4 && kb <= 220) ? (size_t)kb * 1024 : kQrCtaBytes;
   }();
   return lim;
 }
-
-static void qr_smem_attrs() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    const int big = (int)kQrCtaSmem;
-    const int wmax = (int)(8 * kQrWarpSlot);
-    CK(cudaFuncSetAttribute(k_qr_cta<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cta<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cta<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cta<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_warp<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax));
-    CK(cudaFuncSetAttribute(k_qr_warp<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax));
-    CK(cudaFuncSetAttribute(k_qr_warp<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax));
-    CK(cudaFuncSetAttribute(k_qr_warp<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax));
-    CK(cudaFuncSetAttribute(k_qr_cluster<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cluster<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cluster<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    CK(cudaFuncSetAttribute(k_qr_cluster<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  });
-}
-
-// A cluster launch of k_qr_cluster (R CTAs per problem); false when no cluster
-// of that shape and shared memory can be resident (the caller then falls back).
-template <typename TC, bool PIV>
-static bool launch_qr_cluster(const QrcpDesc* d, int nd, int R, size_t smem, cudaStream_t s, bool probe_only) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(nd * R), 1, 1);
-  cfg.blockDim = dim3(512, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)R;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (probe_only) {
-    int ncl = 0;
-    if (cudaOccupancyMaxActiveClusters(&ncl, k_qr_cluster<TC, PIV>, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    return ncl > 0;
-  }
-  CK(cudaLaunchKernelEx(&cfg, k_qr_cluster<TC, PIV>, d, nd));
-  return true;
-}
-
-// Launches problems that all fit in kQrCtaSmem: the warp bucket, then the CTA bucket.
-static constexpr int kQrClusterSizes[3] = {2, 4, 8};
-
-template <bool PIV>
-static void launch_qr_fitting(DescStage& st, const std::vector<QrcpDesc>& v, int prec,
-                              const std::vector<QrcpDesc>* clus = nullptr) {
-  const int tcb = prec == P32 ? 4 : 8;
-  // classes: warp per problem (slot <= kQrWarpSlot), then CTA per problem in
-  // shared-memory size classes (<= 24, 48, 96, 220 KB).  A launch reserves its
-  // largest slot for every CTA, so one large block must not set the occupancy of
-  // many small ones; classes with few CTAs per SM get more threads to hide the
-  // latency of each column step.  The classes run concurrently.
+struct QrPlan {
+  int cls = -1;  // -1: does not fit; kQrClasses, kQrClasses + 1: a warp, 64 / 128 rows
+  int R = 1;     // CTAs per problem, at least
+};
+static QrPlan qr_plan(int m, int n, int tcb) {
+  QrPlan p;
   const size_t lim = qr_cta_limit();
-  const size_t cls[5] = {std::min(kQrWarpSlot, lim), std::min<size_t>(24 * 1024, lim), std::min<size_t>(48 * 1024, lim),
-                         std::min<size_t>(96 * 1024, lim), lim};
-  // (a launch of fewer problems than SMs gives every CTA 1024 threads)
-  const bool few = v.size() < 152;
-  const int thr[5] = {0, few ? 1024 : 256, few ? 1024 : 256, few ? 1024 : 512, 1024};
-  std::vector<QrcpDesc> part[5];
-  size_t smax[5] = {16, 16, 16, 16, 16};
-  for (auto& x : v) {
-    const size_t b = qr_slot_bytes(x.m, x.n, tcb);
-    int c = 0;
-    while (c < 4 && b > cls[c]) ++c;
-    part[c].push_back(x);
-    smax[c] = std::max(smax[c], b);
+  const bool limited = lim < kQrCtaBytes;
+  const size_t bytes = (size_t)m * n * tcb;
+  if (n <= kQrWarpCols && m <= 128 && bytes <= lim) {
+    p.cls = kQrClasses + (m > 64);
+    return p;
   }
-  const QrcpDesc* d[5] = {};
-  for (int c = 0; c < 5; ++c)
-    if (!part[c].empty()) d[c] = st.push(part[c]);
-  const QrcpDesc* dcl[3] = {};
-  size_t scl[3] = {16, 16, 16};
-  for (int c = 0; clus && c < 3; ++c) {
-    if (clus[c].empty()) continue;
-    dcl[c] = st.push(clus[c]);
-    for (auto& x : clus[c]) scl[c] = std::max(scl[c], qr_cluster_slot_bytes(x.m, x.n, kQrClusterSizes[c], tcb));
+  int c = 0;
+  while (c < kQrClasses && m > 32 * kQrRows[c]) ++c;
+  if (c == kQrClasses) return p;
+  const int cols = 16 * qr_class_cols(kQrRows[c], tcb);  // of a CTA of 16 warps
+  const int rmax = limited ? 8 : 16;
+  while (p.R <= rmax && ((size_t)p.R * cols < (size_t)n || (bytes + p.R - 1) / p.R > lim)) p.R *= 2;
+  if (p.R <= rmax) p.cls = c;
+  return p;
+}
+
+static auto qr_launcher(bool piv, int prec) {
+  return prec == P32 ? (piv ? qr_launch_f32_piv : qr_launch_f32_plain)
+                     : (piv ? qr_launch_f64_piv : qr_launch_f64_plain);
+}
+
+// Launches problems that all have a plan.
+template <bool PIV>
+static void launch_qr_fitting(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
+  const int tcb = prec == P32 ? 4 : 8;
+  std::vector<QrcpDesc> warp[2];
+  std::map<std::pair<int, int>, std::vector<QrcpDesc>> part;  // (class, CTAs) -> problems
+  std::vector<QrPlan> plan(v.size());
+  long total = 0;
+  for (size_t i = 0; i < v.size(); ++i) {
+    plan[i] = qr_plan(v[i].m, v[i].n, tcb);
+    if (plan[i].cls < kQrClasses) total += plan[i].R;
   }
+  const int lim = qr_cta_limit() < kQrCtaBytes ? 1 : (tcb == 8 ? 2 * 152 : 152);
+  int mul = 1;
+  while (mul < 16 && total * mul * 2 <= lim) mul *= 2;
+  for (size_t i = 0; i < v.size(); ++i) {
+    const QrPlan& p = plan[i];
+    if (p.cls >= kQrClasses) {
+      warp[p.cls - kQrClasses].push_back(v[i]);
+      continue;
+    }
+    int R = p.R, f = mul;
+    const int cols = qr_class_cols(kQrRows[p.cls], tcb);
+    for (; f > 1 && R * 2 <= 8 && v[i].n >= 4 * cols * R; f /= 2) R *= 2;  // at least two warps per CTA
+    part[{p.cls, R}].push_back(v[i]);
+  }
+  struct Launch {
+    int cls, R, warps;
+    size_t smem;
+    const QrcpDesc* d;
+    int nd;
+  };
+  std::vector<Launch> ls;
+  for (auto& x : part) {
+    Launch l{x.first.first, x.first.second, 1, 0, st.push(x.second), (int)x.second.size()};
+    int nmax = 1;
+    for (auto& y : x.second) nmax = std::max(nmax, y.n);
+    const int cols = qr_class_cols(kQrRows[l.cls], tcb);
+    l.warps = (nmax + cols * l.R - 1) / (cols * l.R);
+    l.smem = qr_reg_bytes(kQrRows[l.cls], nmax, l.warps * l.R, tcb);
+    ls.push_back(l);
+  }
+  const QrcpDesc* dw[2] = {nullptr, nullptr};
+  for (int t = 0; t < 2; ++t)
+    if (!warp[t].empty()) dw[t] = st.push(warp[t]);
   ForkJoin fj(st.stream);
   int li = 0;
-  for (int c = 0; clus && c < 3; ++c) {
-    if (clus[c].empty()) continue;
-    cudaStream_t s = fj.stream(li++);
-    const int nd = (int)clus[c].size();
-    if (prec == P32)
-      launch_qr_cluster<float, PIV>(dcl[c], nd, kQrClusterSizes[c], scl[c], s, false);
-    else
-      launch_qr_cluster<double, PIV>(dcl[c], nd, kQrClusterSizes[c], scl[c], s, false);
-    check_launch("k_qr_cluster");
-    profiler().count(prec == P32 ? KK_QRC32 : KK_QRC64, 1);
+  for (size_t x = ls.size(); x-- > 0;) {  // the tallest first
+    const Launch& l = ls[x];
+    auto go = qr_launcher(PIV, prec);
+    IFMM_REQUIRE(go(l.cls, l.d, l.nd, l.R, l.warps, l.smem, fj.stream(li++), false), IFMM_ECUDA,
+                 "QR launch failed");
+    check_launch("k_qr_reg");
+    if (l.R > 1) profiler().count(prec == P32 ? KK_QRC32 : KK_QRC64, 1);
   }
-  for (int c = 0; c < 5; ++c) {
-    if (part[c].empty()) continue;
-    const int nd = (int)part[c].size();
-    cudaStream_t s = fj.stream(li++);
-    if (c == 0) {
-      // warps per CTA: as many slots as fit in 48 KB, 1..8
-      const int nwp = (int)std::max<size_t>(1, std::min<size_t>(8, (48 * 1024) / smax[0]));
-      const unsigned grid = (unsigned)((nd + nwp - 1) / nwp);
-      const size_t smem = smax[0] * nwp;
-      if (prec == P32)
-        k_qr_warp<float, PIV><<<grid, 32 * nwp, smem, s>>>(d[0], nd, (int)smax[0]);
-      else
-        k_qr_warp<double, PIV><<<grid, 32 * nwp, smem, s>>>(d[0], nd, (int)smax[0]);
-      check_launch("k_qr_warp");
-    } else {
-      if (prec == P32)
-        k_qr_cta<float, PIV><<<(unsigned)nd, thr[c], smax[c], s>>>(d[c], nd);
-      else
-        k_qr_cta<double, PIV><<<(unsigned)nd, thr[c], smax[c], s>>>(d[c], nd);
-      check_launch("k_qr_cta");
-    }
+  for (int t = 1; t >= 0; --t) {
+    if (warp[t].empty()) continue;
+    auto go = prec == P32 ? (PIV ? qr_launch_warp_f32_piv : qr_launch_warp_f32_plain)
+                          : (PIV ? qr_launch_warp_f64_piv : qr_launch_warp_f64_plain);
+    go(t == 1, dw[t], (int)warp[t].size(), fj.stream(li++));
+    check_launch("k_qr_reg");
   }
   fj.join();
 }
 
-// Launches the shared-memory part of a QR batch (reducing tall blocks first);
+// Launches the register-resident part of a QR batch (reducing tall blocks first);
 // returns the indices of the descriptors left for the global-memory kernel.
 template <bool PIV>
-static std::vector<size_t> launch_qr_smem(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
+static std::vector<size_t> launch_qr_reg(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
   const int tcb = prec == P32 ? 4 : 8;
-  const size_t lim = qr_cta_limit();
-  qr_smem_attrs();
   std::vector<QrcpDesc> pre, fit;
   std::vector<size_t> rest;
+  // whether a cluster of R CTAs can be resident (probed once per class and size)
+  static std::mutex mu;
+  static int ok_cache[2][2][kQrClasses][17] = {};  // 0 unknown, 1 yes, -1 no
+  auto resident = [&](const QrPlan& p) {
+    if (p.cls < 0) return false;
+    if (p.cls >= kQrClasses || p.R <= 8) return true;  // portable sizes
+    std::lock_guard<std::mutex> lock(mu);
+    int& ok = ok_cache[prec == P32][PIV][p.cls][p.R];
+    if (!ok) {
+      auto go = qr_launcher(PIV, prec);
+      ok = go(p.cls, nullptr, 1, p.R, 16, qr_reg_bytes(kQrRows[p.cls], 1024, 16 * p.R, tcb), st.stream, true)
+               ? 1 : -1;
+    }
+    return ok > 0;
+  };
   for (size_t i = 0; i < v.size(); ++i) {
     const QrcpDesc& x = v[i];
-    if (qr_slot_bytes(x.m, x.n, tcb) <= lim) {
+    // Tall blocks of 17 to 64 columns (the weight stacks) are reduced by chunks of
+    // 256 rows even where they would fit as a whole: eight rows per lane leave
+    // registers for three times as many problems per SM.  Measured (all QR of one
+    // level): 131,072 points, level 5: 120 -> 71 ms, 8,192 points FP64, level 3:
+    // 124 -> 101; narrower blocks lose (level 6: 18 -> 36 ms).
+    const int tall = x.rb == 0 && x.n > kQrWarpCols && x.n <= 64 && x.m > 384 ? 256 : 0;
+    if (!tall && resident(qr_plan(x.m, x.n, tcb))) {
       fit.push_back(x);
       continue;
     }
-    // largest chunk height c with a fitting slot
-    long c = (long)((lim - sizeof(int) * (size_t)x.n - 16) / tcb) / std::max(1, x.n) - 2;
-    while (c > 0 && qr_slot_bytes((int)c, x.n, tcb) > lim) --c;
-    if (x.rb > 0 || x.m <= x.n || c < x.n) {
+    // else the tallest chunk that has a plan (a multiple of 32 rows)
+    int c = tall ? tall : 32 * kQrRows[kQrClasses - 1];
+    while (c > x.n && !resident(qr_plan(c, x.n, tcb))) c -= 32;
+    if (x.rb > 0 || x.m <= x.n || c <= x.n) {
       rest.push_back(i);
       continue;
     }
-    const int nch = (int)((x.m + c - 1) / c);
-    const int last = x.m - (nch - 1) * (int)c;
+    const int nch = (x.m + c - 1) / c;
+    const int last = x.m - (nch - 1) * c;
     const int mv = (nch - 1) * x.n + std::min(x.n, last);
-    if (qr_slot_bytes(mv, x.n, tcb) > lim) {
+    if (!resident(qr_plan(mv, x.n, tcb))) {
       rest.push_back(i);
       continue;
     }
@@ -674,48 +664,19 @@ static std::vector<size_t> launch_qr_smem(DescStage& st, const std::vector<QrcpD
       QrcpDesc q{};
       q.A = x.A + (long)j * c;
       q.ld = x.ld;
-      q.m = std::min((int)c, x.m - j * (int)c);
+      q.m = std::min(c, x.m - j * c);
       q.n = x.n;
       pre.push_back(q);
     }
     QrcpDesc y = x;
     y.m = mv;
     y.rb = x.n;
-    y.rs = (int)c;
+    y.rs = c;
     fit.push_back(y);
   }
-  // what neither fits nor reduces goes to a cluster of 2, 4 or 8 CTAs when its
-  // rows fit their shared memory (rows addressed plainly: rb == 0)
-  std::vector<QrcpDesc> clus[3];
-  std::vector<size_t> left;
-  for (size_t i : rest) {
-    const QrcpDesc& x = v[i];
-    int c = -1;
-    if (x.rb == 0)
-      for (int q = 0; q < 3 && c < 0; ++q)
-        if (qr_cluster_slot_bytes(x.m, x.n, kQrClusterSizes[q], tcb) <= lim) c = q;
-    if (c >= 0) {
-      // residency of the largest cluster slot of each size (probed once)
-      static std::mutex mu;
-      static int ok_cache[2][2][3] = {};  // 0 unknown, 1 yes, -1 no
-      int& ok = ok_cache[prec == P32 ? 0 : 1][PIV ? 1 : 0][c];
-      std::lock_guard<std::mutex> lock(mu);
-      if (ok == 0) {
-        const bool r = prec == P32
-                           ? launch_qr_cluster<float, PIV>(nullptr, 1, kQrClusterSizes[c], kQrCtaSmem, st.stream, true)
-                           : launch_qr_cluster<double, PIV>(nullptr, 1, kQrClusterSizes[c], kQrCtaSmem, st.stream, true);
-        ok = r ? 1 : -1;
-      }
-      if (ok < 0) c = -1;
-    }
-    if (c >= 0)
-      clus[c].push_back(x);
-    else
-      left.push_back(i);
-  }
   if (!pre.empty()) launch_qr_fitting<false>(st, pre, prec);
-  launch_qr_fitting<PIV>(st, fit, prec, clus);
-  return left;
+  if (!fit.empty()) launch_qr_fitting<PIV>(st, fit, prec);
+  return rest;
 }
 
 void launch_qr(DescStage& st, const std::vector<QrDesc>& v, int prec) {
@@ -737,7 +698,7 @@ void launch_qr(DescStage& st, const std::vector<QrDesc>& v, int prec) {
     q.n = v[i].n;
     as[i] = q;
   }
-  const std::vector<size_t> rest = launch_qr_smem<false>(st, as, prec);
+  const std::vector<size_t> rest = launch_qr_reg<false>(st, as, prec);
   profiler().end(kk, st.stream, pe);
   if (!rest.empty()) {
     std::vector<QrDesc> g;
@@ -772,7 +733,7 @@ void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
   prof_batch_tag() = (long)v.size();
   const int kk = prec == P32 ? KK_QR32 : KK_QR64;
   cudaEvent_t pe = profiler().begin(kk, st.stream);
-  const std::vector<size_t> rest = launch_qr_smem<true>(st, v, prec);
+  const std::vector<size_t> rest = launch_qr_reg<true>(st, v, prec);
   profiler().end(kk, st.stream, pe);
   if (!rest.empty()) {
     std::vector<QrcpDesc> g;
