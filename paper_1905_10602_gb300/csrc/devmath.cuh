@@ -61,6 +61,14 @@ __device__ __forceinline__ double f2d_pow2(float f, int sh) {
 // biased binary64 exponent of |d| (0 for zero and subnormals, 2047 for inf/NaN)
 __device__ __forceinline__ int dexp(double d) { return (int)(((unsigned)__double2hiint(d) & 0x7fffffffu) >> 20); }
 
+// d times 2^sh by its exponent field; results outside the normal range by ldexp
+static __device__ __noinline__ double ldexp_rare(double d, int sh) { return ldexp(d, sh); }
+__device__ __forceinline__ double scale_pow2(double d, int sh) {
+  const int e = dexp(d);
+  if (d == 0.0 || e == 2047) return d;
+  if (e == 0 || e + sh <= 0 || e + sh >= 2047) return ldexp_rare(d, sh);
+  return __hiloint2double(__double2hiint(d) + (sh << 20), __double2loint(d));
+}
 // value of a double as the arithmetic type TC, times 2^sh
 template <typename TC>
 __device__ __forceinline__ TC ld_tc(double d, int sh = 0) {

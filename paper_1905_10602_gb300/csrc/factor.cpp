@@ -1803,12 +1803,13 @@ struct Factorizer {
     F.ntop = nt;
     F.top_inv = F.persist.alloc((size_t)std::max(1, nt) * std::max(1, nt));
     if (!nt) return;
+    double* M = scratch().alloc((size_t)nt * nt);
     std::vector<CopyDesc> cc;
     for (int a = 0; a < W.nn; ++a)
       for (int b = 0; b < W.nn; ++b) {
         if (!W.r[a] || !W.r[b]) continue;
         const int sl = W.slot(a, b);
-        double* dst = F.top_inv + F.top_off[a] + (long)F.top_off[b] * nt;
+        double* dst = M + F.top_off[a] + (long)F.top_off[b] * nt;
         if (sl >= 0) {
           cc.push_back(cpy(W.nb[2][sl], W.n[a], dst, nt, W.r[a], W.r[b]));
         } else {
@@ -1819,10 +1820,10 @@ struct Factorizer {
       }
     (void)LL;
     launch_copy(st, cc);
-    double* wk = scratch().alloc(2 * (size_t)nt);
+    double* wk = scratch().alloc(big_inverse_work_doubles(nt));
     int* wi = (int*)scratch().alloc((size_t)nt);
     int* info = (int*)scratch().alloc(1);
-    big_inverse(s, F.top_inv, nt, nt, wi, wk, info);
+    big_inverse(s, M, nt, F.top_inv, wi, wk, info);
     cnt.lu += 2.0 * std::pow((double)nt, 3);
     int hinfo = 0;
     CK(cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -32,14 +32,6 @@
 
 namespace ifmm {
 
-// d times 2^sh by its exponent field; results outside the normal range by ldexp
-static __device__ __noinline__ double ldexp_rare(double d, int sh) { return ldexp(d, sh); }
-__device__ __forceinline__ double scale_pow2(double d, int sh) {
-  const int e = dexp(d);
-  if (d == 0.0 || e == 2047) return d;
-  if (e == 0 || e + sh <= 0 || e + sh >= 2047) return ldexp_rare(d, sh);
-  return __hiloint2double(__double2hiint(d) + (sh << 20), __double2loint(d));
-}
 // An element of the block between its conversions: the FP64 slot, or its first half
 // when the arithmetic is FP32.  The conversions are long integer sequences, so they
 // stand in two short loops (in, out) over the block in global memory, and the

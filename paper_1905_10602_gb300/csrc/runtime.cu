@@ -10,6 +10,7 @@
 #include "pairs.cuh"
 #include "matvec_fp64.cuh"
 #include "krylov.cuh"
+#include "biginv.cuh"
 #include "ifmm_kernels.h"
 #include "qr.h"
 #include "runtime.h"
@@ -2022,17 +2023,92 @@ __global__ void k_gj_colswap(double* A, long ld, int n, const int* piv, const in
   }
 }
 
-void big_inverse(cudaStream_t s, double* A, int ld, int n, int* d_work_int, double* d_work, int* d_info) {
-  // d_work_int: n ints (pivots); d_work: 2n doubles; d_info: 1 int (zeroed here)
-  CK(cudaMemsetAsync(d_info, 0, sizeof(int), s));
+// The two launches per column, in place, for matrices whose panels fit no cluster.
+static void big_inverse_columns(cudaStream_t s, double* A, int ld, int n, int* d_piv, double* d_work, int* d_info) {
   const int upd_blocks = (int)std::max<long>(1, std::min<long>(152L * 8, ((long)n * ((n + 255) / 256) + 7) / 8));
-  cudaEvent_t pe = profiler().begin(KK_GJ_BIG, s, 2L * n + 1);
   for (int k = 0; k < n; ++k) {
-    k_gj_pivot<<<1, 1024, 0, s>>>(A, ld, n, k, d_work_int, d_work, d_work + n, d_info);
+    k_gj_pivot<<<1, 1024, 0, s>>>(A, ld, n, k, d_piv, d_work, d_work + n, d_info);
     k_gj_update<<<upd_blocks, 256, 0, s>>>(A, ld, n, k, d_work, d_work + n, d_info);
   }
-  k_gj_colswap<<<1, 1024, 0, s>>>(A, ld, n, d_work_int, d_info);
+  k_gj_colswap<<<1, 1024, 0, s>>>(A, ld, n, d_piv, d_info);
   check_launch("big_inverse", 2L * n + 1);
+}
+
+size_t big_inverse_work_doubles(int n) { return std::max((bi_work_bytes(n) + 7) / 8, (size_t)2 * n); }
+
+void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, double* d_work, int* d_info) {
+  CK(cudaMemsetAsync(d_info, 0, sizeof(int), s));
+  // CTAs of the panel's cluster: rows of at most two per thread and what shared
+  // memory holds; 16 (a non-portable size) when the GPU can host it and the
+  // matrix has rows enough for them
+  static std::once_flag once;
+  static int rmax = 0;
+  std::call_once(once, [] {
+    CK(cudaFuncSetAttribute(k_bi_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    CK(cudaFuncSetAttribute(k_bi_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kBiGemmBytes));
+    rmax = 8;
+    if (cudaFuncSetAttribute(k_bi_panel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+      cudaGetLastError();
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(16);
+    c.blockDim = dim3(kBiThreads);
+    c.dynamicSmemBytes = 220 * 1024;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 16;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    int ncl = 0;
+    if (cudaOccupancyMaxActiveClusters(&ncl, k_bi_panel, &c) == cudaSuccess && ncl > 0)
+      rmax = 16;
+    else
+      cudaGetLastError();
+  });
+  int R = 1;
+  while (R < rmax && bi_rows(n, R) > 32) R *= 2;
+  cudaEvent_t pe = profiler().begin(KK_GJ_BIG, s, 1);
+  if (bi_rows(n, R) > 2 * kBiThreads || bi_panel_bytes(n, R) > (size_t)220 * 1024) {
+    big_inverse_columns(s, M, n, n, d_piv, d_work, d_info);
+    CK(cudaMemcpyAsync(out, M, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
+    profiler().end(KK_GJ_BIG, s, pe);
+    return;
+  }
+  BiWork w;
+  w.np = (n + kBiTile - 1) / kBiTile * kBiTile;
+  w.da = (uint16_t*)d_work;
+  w.db = w.da + (size_t)kBiSlices * w.np * kBiNb;
+  w.ea = (int*)(w.db + (size_t)kBiSlices * w.np * kBiNb);
+  w.eb = w.ea + w.np;
+  w.used = (unsigned char*)(w.eb + w.np);
+  CK(cudaMemsetAsync(w.used, 0, w.np, s));
+  CK(cudaMemsetAsync(w.da, 0, sizeof(uint16_t) * (size_t)kBiSlices * w.np * kBiNb, s));  // the padding rows
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)R);
+  cfg.blockDim = dim3(kBiThreads);
+  cfg.dynamicSmemBytes = bi_panel_bytes(n, R);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)R;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const unsigned tiles = (unsigned)(w.np / kBiTile);
+  long launches = 0;
+  for (int k0 = 0; k0 < n; k0 += kBiNb) {
+    const int kb = std::min(kBiNb, n - k0);
+    CK(cudaLaunchKernelEx(&cfg, k_bi_panel, M, n, k0, kb, d_piv, w, d_info));
+    ++launches;
+    if (n > kb) {
+      k_bi_rows<<<(unsigned)(w.np / 8), 256, 0, s>>>(M, n, k0, kb, d_piv, w, d_info);
+      k_bi_gemm<<<dim3(tiles, tiles), 128, kBiGemmBytes, s>>>(M, n, w, d_info);
+      launches += 2;
+    }
+  }
+  k_bi_out<<<dim3((unsigned)((n + 255) / 256), (unsigned)std::min(n, 4096)), 256, 0, s>>>(M, n, d_piv, out, n, d_info);
+  check_launch("big_inverse", launches + 1);
+  profiler().count(KK_GJ_BIG, launches);
   profiler().end(KK_GJ_BIG, s, pe);
 }
 
