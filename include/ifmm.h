@@ -145,7 +145,8 @@ ifmm_status ifmm_color_levels(ifmm_tree* t, int sigma, int tau, int32_t* ncolors
  *   "perm"            tree order -> caller index (level ignored)
  *   "leaf_ptr"        point CSR of the leaves (level ignored)
  *   "matvec_block"    2 values: the source tile (threads per CTA) and the targets
- *                     per thread of the float-pair matvec, chosen by its autotuner
+ *                     per thread of the float-pair matvec (128 or 256, and 3: the
+ *                     tiles of the symmetric kernel), chosen by its autotuner
  *                     on the first such product with this tree (0, 0 before); the
  *                     choice is remembered per device and N for the life of the
  *                     process, and trees of a size tuned before reuse it

@@ -52,6 +52,21 @@ __device__ __forceinline__ df df_rsqrt_fast(df x) {
   const float e = (1.f - uh) - ul;
   return {y0, 0.5f * y0 * e};
 }
+// |d|^2 of d = (x, y, z): with the largest high part squared first, each partial
+// sum s' = fma(h, h, s) is at most twice s, so that s - s' is exact and one FMA
+// gives the rounding error of the step (8 operations instead of three squares as
+// pairs and two two-sums, 18); the low parts' products as in df_sq.
+__device__ __forceinline__ df df_norm2(df x, df y, df z) {
+  const float a = fabsf(x.h), b = fabsf(y.h), c = fabsf(z.h);
+  const float hi = fmaxf(a, b), lo = fminf(a, b);
+  const float m = fmaxf(hi, c), o = fminf(hi, c);
+  const float p = m * m, e1 = fmaf(m, m, -p);
+  const float s = fmaf(o, o, p), e2 = fmaf(o, o, p - s);
+  const float t = fmaf(lo, lo, s), e3 = fmaf(lo, lo, s - t);
+  const float cr = fmaf(x.h, x.l, fmaf(y.h, y.l, z.h * z.l));
+  const float ll = fmaf(x.l, x.l, fmaf(y.l, y.l, z.l * z.l));
+  return df_quick(t, fmaf(2.f, cr, ll) + (e1 + (e2 + e3)));
+}
 // acc + (ph + pl): two-sum of the high parts, low parts added
 __device__ __forceinline__ df df_acc(df acc, float ph, float pl) {
   const df s = df_two_sum(acc.h, ph);

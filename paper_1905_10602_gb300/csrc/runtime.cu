@@ -1468,24 +1468,26 @@ __global__ void __launch_bounds__(BS) k_matvec_df(const float* __restrict__ pts,
 
 // The same sum with each unordered pair (i, j), i != j, evaluated once: the
 // kernel is symmetric (1/|x_i - x_j|), so one 1/r serves both q_j / r (row i)
-// and q_i / r (row j).  The points are cut into tiles of kSymTile; a CTA takes
-// one pair of tiles (I <= J): every warp holds 32 targets of tile I and walks
-// the 128 sources of tile J in four chunks of 32, lane l meeting source
-// (l + step) mod 32 of the chunk at each step, so that the 32 lanes touch 32
-// different sources and add their q_i / r into per-warp shared-memory column
-// sums without atomics (a __syncwarp between steps orders them).  Each CTA
+// and q_i / r (row j).  The points are cut into tiles of TB = 128 TPT; a CTA of
+// 128 threads takes one pair of tiles (I <= J): every warp holds 32 TPT targets
+// of tile I, TPT per lane, and walks the sources of tile J in chunks of 32, lane l
+// meeting source (l + step) mod 32 of the chunk at each step, so that the 32 lanes
+// touch 32 different sources and add their q_i / r into per-warp shared-memory
+// column sums without atomics (a __syncwarp between steps orders them).  Each CTA
 // writes its row sums as tile J's partial of the targets and its column sums,
 // combined over the warps in a fixed order, as tile I's partial of the sources:
 // part[B * n + p] is tile B's contribution to point p, written exactly once.  A
 // diagonal tile (I == J) takes every ordered pair once, rows only.  The second
 // kernel adds the T partials of each point in tile order.  Both orders are
 // fixed, so the result does not depend on scheduling.
-constexpr int kSymTile = 128;
+//
+// Bound: the FP32 issue rate.  TPT = 2 halves the shared-memory accesses, the
+// barrier and the loop per pair and gives two independent chains; the squared
+// distance takes 25 operations (df_norm2; 37 before).  One product at n = 131,072:
+// 28.9 ms -> 24.6.  The autotuner keeps TPT = 1 where tiles of 256 are too few.
+constexpr int kSymThreads = 128;
 __device__ __forceinline__ df sym_w(df px, df py, df pz, float4 a, float4 b) {
-  const df dx = df_diff(px, a.x, a.y);
-  const df dy = df_diff(py, a.z, a.w);
-  const df dz = df_diff(pz, b.x, b.y);
-  return df_rsqrt_fast(df_sum3(df_sq(dx), df_sq(dy), df_sq(dz)));
+  return df_rsqrt_fast(df_norm2(df_diff(px, a.x, a.y), df_diff(py, a.z, a.w), df_diff(pz, b.x, b.y)));
 }
 // q w as a pair added to acc (q a pair, w a pair)
 __device__ __forceinline__ df sym_add(df acc, float qh, float ql, df w) {
@@ -1493,21 +1495,16 @@ __device__ __forceinline__ df sym_add(df acc, float qh, float ql, df w) {
   const float pl = fmaf(qh, w.h, -ph) + fmaf(qh, w.l, ql * w.h);
   return df_acc(acc, ph, pl);
 }
-__global__ void __launch_bounds__(kSymTile) k_matvec_sym(const float* __restrict__ pts, const float* __restrict__ qh,
-                                                         const float* __restrict__ ql, int n, int T,
-                                                         float2* __restrict__ part) {
-  constexpr int TB = kSymTile;
+template <int TPT>
+__global__ void __launch_bounds__(kSymThreads) k_matvec_sym(const float* __restrict__ pts,
+                                                            const float* __restrict__ qh,
+                                                            const float* __restrict__ ql, int n, int T,
+                                                            float2* __restrict__ part) {
+  constexpr int TB = kSymThreads * TPT, NW = kSymThreads / 32;
   __shared__ float4 sa[TB], sb[TB];
-  __shared__ float2 col[TB / 32][TB];
-  // tile pair of this CTA: b = I T - I (I - 1) / 2 + (J - I), I <= J
-  const long bid = blockIdx.x;
-  int I = (int)((2.0 * T + 1.0 - sqrt((2.0 * T + 1.0) * (2.0 * T + 1.0) - 8.0 * (double)bid)) / 2.0);
-  auto first = [&](int i) { return (long)i * T - (long)i * (i - 1) / 2; };
-  if (I < 0) I = 0;
-  if (I > T - 1) I = T - 1;
-  while (I > 0 && first(I) > bid) --I;
-  while (I < T - 1 && first(I + 1) <= bid) ++I;
-  const int J = I + (int)(bid - first(I));
+  __shared__ float2 col[NW][TB];
+  int I, J;
+  tile_pair(blockIdx.x, T, &I, &J);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const float* xh = pts;
   const float* xl = pts + n;
@@ -1517,55 +1514,83 @@ __global__ void __launch_bounds__(kSymTile) k_matvec_sym(const float* __restrict
   const float* zl = pts + 5 * (long)n;
   // outside the points: far away (finite distances) with zero charge
   constexpr float kFar = 1e15f;
-  const int i = I * TB + tid, j = J * TB + tid;
-  df px = {kFar, 0.f}, py = {kFar, 0.f}, pz = {kFar, 0.f};
-  float qih = 0.f, qil = 0.f;
-  if (i < n) {
-    px = {xh[i], xl[i]};
-    py = {yh[i], yl[i]};
-    pz = {zh[i], zl[i]};
-    qih = qh[i];
-    qil = ql[i];
-  }
-  if (j < n) {
-    sa[tid] = make_float4(xh[j], xl[j], yh[j], yl[j]);
-    sb[tid] = make_float4(zh[j], zl[j], qh[j], ql[j]);
-  } else {
-    sa[tid] = make_float4(-kFar, 0.f, -kFar, 0.f);
-    sb[tid] = make_float4(-kFar, 0.f, 0.f, 0.f);
+  df px[TPT], py[TPT], pz[TPT], acc[TPT];
+  float qih[TPT], qil[TPT];
+  int ti[TPT];  // the lane's targets in tile I
+#pragma unroll
+  for (int u = 0; u < TPT; ++u) {
+    ti[u] = w * 32 * TPT + u * 32 + lane;
+    const int i = I * TB + ti[u];
+    px[u] = py[u] = pz[u] = {kFar, 0.f};
+    acc[u] = {0.f, 0.f};
+    qih[u] = qil[u] = 0.f;
+    if (i < n) {
+      px[u] = {xh[i], xl[i]};
+      py[u] = {yh[i], yl[i]};
+      pz[u] = {zh[i], zl[i]};
+      qih[u] = qh[i];
+      qil[u] = ql[i];
+    }
   }
 #pragma unroll
-  for (int u = 0; u < TB / 32; ++u) col[u][tid] = make_float2(0.f, 0.f);
+  for (int u = 0; u < TPT; ++u) {
+    const int s = tid + u * kSymThreads, j = J * TB + s;
+    if (j < n) {
+      sa[s] = make_float4(xh[j], xl[j], yh[j], yl[j]);
+      sb[s] = make_float4(zh[j], zl[j], qh[j], ql[j]);
+    } else {
+      sa[s] = make_float4(-kFar, 0.f, -kFar, 0.f);
+      sb[s] = make_float4(-kFar, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int x = 0; x < NW; ++x) col[x][s] = make_float2(0.f, 0.f);
+  }
   __syncthreads();
-  df acc = {0.f, 0.f};
   if (I == J) {
     for (int t = 0; t < TB; ++t) {
       const float4 a = sa[t], b = sb[t];
-      const df wr = sym_w(px, py, pz, a, b);
-      if (t != tid) acc = sym_add(acc, b.z, b.w, wr);
+#pragma unroll
+      for (int u = 0; u < TPT; ++u) {
+        const df wr = sym_w(px[u], py[u], pz[u], a, b);
+        if (t != ti[u]) acc[u] = sym_add(acc[u], b.z, b.w, wr);
+      }
     }
   } else {
     float2* mycol = col[w];
     for (int c = 0; c < TB; c += 32) {
+#pragma unroll 2
       for (int r = 0; r < 32; ++r) {
         const int sidx = c + ((lane + r) & 31);
         const float4 a = sa[sidx], b = sb[sidx];
-        const df wr = sym_w(px, py, pz, a, b);
-        acc = sym_add(acc, b.z, b.w, wr);
+        df wr[TPT];
+#pragma unroll
+        for (int u = 0; u < TPT; ++u) {
+          wr[u] = sym_w(px[u], py[u], pz[u], a, b);
+          acc[u] = sym_add(acc[u], b.z, b.w, wr[u]);
+        }
         const float2 cv = mycol[sidx];
-        const df cs = sym_add({cv.x, cv.y}, qih, qil, wr);
+        df cs = {cv.x, cv.y};
+#pragma unroll
+        for (int u = 0; u < TPT; ++u) cs = sym_add(cs, qih[u], qil[u], wr[u]);
         mycol[sidx] = make_float2(cs.h, cs.l);
         __syncwarp();
       }
     }
   }
-  if (i < n) part[(long)J * n + i] = make_float2(acc.h, acc.l);
+#pragma unroll
+  for (int u = 0; u < TPT; ++u) {
+    const int i = I * TB + ti[u];
+    if (i < n) part[(long)J * n + i] = make_float2(acc[u].h, acc[u].l);
+  }
   if (I != J) {
     __syncthreads();
-    if (j < n) {
-      df cs = {col[0][tid].x, col[0][tid].y};
 #pragma unroll
-      for (int u = 1; u < TB / 32; ++u) cs = df_acc(cs, col[u][tid].x, col[u][tid].y);
+    for (int u = 0; u < TPT; ++u) {
+      const int s = tid + u * kSymThreads, j = J * TB + s;
+      if (j >= n) continue;
+      df cs = {col[0][s].x, col[0][s].y};
+#pragma unroll
+      for (int x = 1; x < NW; ++x) cs = df_acc(cs, col[x][s].x, col[x][s].y);
       part[(long)I * n + j] = make_float2(cs.h, cs.l);
     }
   }
@@ -1582,9 +1607,10 @@ __global__ void k_matvec_sym_sum(const float2* __restrict__ part, int n, int T, 
   y[p] = diag * x[p] + scale * ((double)acc.h + (double)acc.l);
 }
 
-// floats of partial sums the symmetric float-pair matvec needs for n points
+// floats of partial sums the symmetric float-pair matvec needs for n points (the
+// smaller tile's)
 size_t matvec_sym_part_floats(int n) {
-  const long T = (n + kSymTile - 1) / kSymTile;
+  const long T = (n + kSymThreads - 1) / kSymThreads;
   return (size_t)T * (size_t)n * 2;
 }
 
@@ -1767,13 +1793,17 @@ void launch_split_df(cudaStream_t s, const double* in, float* hi, float* lo, int
   check_launch("k_split_df");
 }
 
-// the tile code: BS | TPT << 16; TPT = 3 is the symmetric kernel (part != NULL)
+// the tile code: BS | TPT << 16; TPT = 3 is the symmetric kernel (part != NULL) with
+// tiles of BS = 128 or 256 points
 static void matvec_df_bs(int code, cudaStream_t s, const float* pts_df, const float* qh, const float* ql,
                          const double* x, double* y, int N, double scale, double diag, float2* part) {
   const int bs = code & 0xffff, tpt = code >> 16;
   if (tpt == 3 && part) {
-    const long T = (N + kSymTile - 1) / kSymTile;
-    k_matvec_sym<<<(unsigned)(T * (T + 1) / 2), kSymTile, 0, s>>>(pts_df, qh, ql, N, (int)T, part);
+    const long T = (N + bs - 1) / bs;
+    if (bs == 2 * kSymThreads)
+      k_matvec_sym<2><<<(unsigned)(T * (T + 1) / 2), kSymThreads, 0, s>>>(pts_df, qh, ql, N, (int)T, part);
+    else
+      k_matvec_sym<1><<<(unsigned)(T * (T + 1) / 2), kSymThreads, 0, s>>>(pts_df, qh, ql, N, (int)T, part);
     k_matvec_sym_sum<<<(N + 255) / 256, 256, 0, s>>>(part, N, (int)T, x, y, scale, diag);
   } else if (tpt == 2) {
     if (bs == 128)
@@ -1795,10 +1825,15 @@ static void matvec_df_bs(int code, cudaStream_t s, const float* pts_df, const fl
 // BS | TPT << 16; y is overwritten.
 int autotune_matvec_df(cudaStream_t s, const float* pts_df, const float* qh, const float* ql, const double* x,
                        double* y, int N, double scale, double diag, float2* part) {
-  std::vector<int> cand = {128 | 1 << 16, 256 | 1 << 16, 512 | 1 << 16, 128 | 2 << 16, 256 | 2 << 16};
-  if (part) cand.push_back(kSymTile | 3 << 16);
+  std::vector<int> cand;
+  if (part) cand = {kSymThreads | 3 << 16, 2 * kSymThreads | 3 << 16};
+  // the full sums do twice the symmetric kernel's work (n = 131,072: 54 against 29
+  // ms) and have CTAs enough for the chip only above 2,048 points: below, or
+  // without its buffer, they are timed too
+  if (!part || N <= 2048)
+    for (int c : {128 | 1 << 16, 256 | 1 << 16, 512 | 1 << 16, 128 | 2 << 16, 256 | 2 << 16}) cand.push_back(c);
   float best = 1e30f;
-  int pick = 256 | 1 << 16;
+  int pick = cand[0];
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
   CK(cudaEventCreate(&b));
@@ -1817,7 +1852,7 @@ int autotune_matvec_df(cudaStream_t s, const float* pts_df, const float* qh, con
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  check_launch("autotune_matvec_df", 9);
+  check_launch("autotune_matvec_df", 3L * (long)cand.size());
   return pick;
 }
 

@@ -338,12 +338,14 @@ static int matvec_tile(ifmm_tree* tm, cudaStream_t s, const float* q, const doub
   std::lock_guard<std::mutex> lock(g_tune_mutex);
   if (tm->matvec_block) return tm->matvec_block;
   // IFMM_MATVEC_TILE (read when a tree first needs its tile) forces a kernel:
-  // "sym", or "<threads>x<targets per thread>" (128x1, 256x1, 512x1, 128x2,
+  // "sym" or "sym2" (tiles of 128 or 256 points), or "<threads>x<targets per thread>" (128x1, 256x1, 512x1, 128x2,
   // 256x2); for tests and experiments
   if (const char* e = getenv("IFMM_MATVEC_TILE")) {
     int code = 0, bs = 0, tpt = 0;
     if (std::string(e) == "sym" && part)
       code = 128 | 3 << 16;
+    else if (std::string(e) == "sym2" && part)
+      code = 256 | 3 << 16;
     else if (sscanf(e, "%dx%d", &bs, &tpt) == 2 && (tpt == 1 || tpt == 2) &&
              (bs == 128 || bs == 256 || (bs == 512 && tpt == 1)))
       code = bs | tpt << 16;
