@@ -35,7 +35,7 @@ struct LevelFactor {
 // either way).  The blocks the solve reads are packed row-major in `mem`.
 struct SolveLaunch {
   const SolveOp* ops;
-  const int* warp_ptr;  // prefix sums of the warps of each op
+  const int2* warps;  // (op, first row) of every warp
   int nops, nwarps;
 };
 

@@ -68,8 +68,11 @@ void launch_zgather(DescStage& st, const std::vector<ZGatherDesc>& v, const ZTab
 // Schur-complement blocks of the eliminated nodes added into their near blocks
 void launch_schur_scatter(DescStage& st, const std::vector<ScatterDesc>& v, const ScatterTables& t, int maxdeg);
 void launch_copy_dev(cudaStream_t s, const CopyDesc* d, int n);
-// the solve's row operations (pairs: float-pair vectors and FP32 matrices)
-void launch_solve_ops(cudaStream_t s, const SolveOp* ops, const int* warp_ptr, int nops, int nwarps, bool pairs);
+// the solve's row operations (pairs: float-pair vectors and FP32 matrices) on nr
+// (1, 2 or 4) vector buffers: every vector pointer of the ops plus off + r stride
+// bytes, r < nr; warps: (op, first row) of every warp
+void launch_solve_ops(cudaStream_t s, const SolveOp* ops, const int2* warps, int nwarps, bool pairs, int nr = 1,
+                      long off = 0, long stride = 0);
 // column-major FP64 blocks -> row-major FP64 / FP32 copies
 void launch_pack(DescStage& st, const std::vector<PackDesc>& v, bool fp32);
 // FP64 <-> float pairs (hi = nearest float, lo = nearest float of the rest)

@@ -5,6 +5,7 @@
 #include <cstring>
 #include <mutex>
 #include <thread>
+#include <type_traits>
 
 #include "dense.cuh"
 #include "pairs.cuh"
@@ -1617,98 +1618,117 @@ size_t matvec_sym_part_floats(int n) {
 // ---------------------------------------------------------------- the solve's row operations
 // out[r] = beta base[r] + alpha sum_c M[r][c] v(c) for the rows of every op of a
 // launch.  `lanes` lanes share a row: each reads 16-byte vectors of the row
-// (4 FP32 or 2 FP64 coefficients) at a stride of lanes vectors, two vectors per
-// step, and the partial sums are combined by shuffles in a fixed order.  A warp
-// covers 32 / lanes rows of one op; warp_ptr gives each op's first warp.
+// (4 FP32 or 2 FP64 coefficients) at a stride of lanes vectors, and the partial
+// sums are combined by shuffles in a fixed order.  A warp covers 32 / lanes rows of
+// one op.
 // PAIRS: FP32 coefficients, float-pair vectors and accumulation (the product of
 // an exact float by a pair is formed with FMAs, so the operator applied is the
 // stored FP32 matrix to ~2^-44); otherwise FP64 throughout.
+//
+// Bound: a program of a few hundred dependent launches, so the latency of each.  A
+// warp finds its op and row in one table entry (a binary search over the ops'
+// first warps took up to a dozen dependent loads); the launches are programmatic
+// dependents of each other, and what the previous one does not write -- table, op,
+// gather indices and the first two vectors of the row -- is loaded before waiting
+// for it.  NR right-hand sides share one reading of the coefficients.  FP64 factor
+// of 12,289 points, one right-hand side in a graph: 2.3 ms -> 1.15; four: 9.6 ms -> 3.8.
 // s + a v(c) with a exact and v(c) a pair: the FMA two-product of a and the
 // high part plus a times the low part, added with a two-sum
-__device__ __forceinline__ df pair_term(df s, float a, const float2* __restrict__ X, const int* __restrict__ xidx,
-                                        int c) {
-  const float2 xv = xidx ? X[xidx[c]] : X[c];
+__device__ __forceinline__ df pair_term(df s, float a, float2 xv) {
   const float p = a * xv.x;
   return df_acc(s, p, fmaf(a, xv.y, fmaf(a, xv.x, -p)));
 }
-template <bool PAIRS>
-__global__ void __launch_bounds__(256) k_solve_rows(const SolveOp* __restrict__ ops, const int* __restrict__ warp_ptr,
-                                                    int nops) {
+template <bool PAIRS, int NR>
+__global__ void __launch_bounds__(256) k_solve_rows(const SolveOp* __restrict__ ops, const int2* __restrict__ warps,
+                                                    int nwarps, long off, long stride) {
+  using T = typename std::conditional<PAIRS, float2, double>::type;  // a vector element
+  using C = typename std::conditional<PAIRS, float, double>::type;   // a coefficient
+  constexpr int VW = 16 / sizeof(C);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int gw = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  if (gw >= warp_ptr[nops]) return;  // whole warps
-  const int oi = find_desc(warp_ptr, nops, gw);
-  const SolveOp& O = ops[oi];
+  if (gw >= nwarps) return;  // whole warps
+  const int2 wt = warps[gw];
+  const SolveOp& O = ops[wt.x];
   const int lane = threadIdx.x & 31;
   const int G = O.lanes;
   const int sub = lane & (G - 1);
-  const int r = (gw - warp_ptr[oi]) * (32 / G) + lane / G;
+  const int r = wt.y + lane / G;
   const bool live = r < O.rows;
   const int nc = live ? O.ncols : 0;
-  if constexpr (PAIRS) {
-    const float2* X = (const float2*)O.x;
-    const int* xi = O.xidx;
-    const float* row = (const float*)O.M + (long)r * O.ldm;
-    df s = {0.f, 0.f};
-    int c = sub * 4;
-    for (; c + G * 4 < nc; c += 2 * G * 4) {
-      const float4 u = *(const float4*)(row + c);
-      const float4 w = *(const float4*)(row + c + G * 4);
-      const int c2 = c + G * 4;
-      s = pair_term(s, u.x, X, xi, c);
-      if (c + 1 < nc) s = pair_term(s, u.y, X, xi, c + 1);
-      if (c + 2 < nc) s = pair_term(s, u.z, X, xi, c + 2);
-      if (c + 3 < nc) s = pair_term(s, u.w, X, xi, c + 3);
-      s = pair_term(s, w.x, X, xi, c2);
-      if (c2 + 1 < nc) s = pair_term(s, w.y, X, xi, c2 + 1);
-      if (c2 + 2 < nc) s = pair_term(s, w.z, X, xi, c2 + 2);
-      if (c2 + 3 < nc) s = pair_term(s, w.w, X, xi, c2 + 3);
-    }
+  const int* xi = O.xidx;
+  const char* X = (const char*)O.x + off;
+  const C* row = (const C*)O.M + (long)r * O.ldm;
+  struct Vec {
+    C v[VW];
+    int i[VW];
+  };
+  auto load = [&](int c) {
+    Vec u;
     if (c < nc) {
-      const float4 u = *(const float4*)(row + c);
-      s = pair_term(s, u.x, X, xi, c);
-      if (c + 1 < nc) s = pair_term(s, u.y, X, xi, c + 1);
-      if (c + 2 < nc) s = pair_term(s, u.z, X, xi, c + 2);
-      if (c + 3 < nc) s = pair_term(s, u.w, X, xi, c + 3);
+      const float4 q = *(const float4*)(row + c);
+      memcpy(u.v, &q, 16);
     }
-    for (int o = G >> 1; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, s.h, o), ol = __shfl_xor_sync(0xffffffffu, s.l, o);
-      s = df_acc(s, oh, ol);
-    }
-    if (live && sub == 0) {
-      const int orow = O.oidx ? O.oidx[r] : r;
-      if (O.alpha < 0.0) s = {-s.h, -s.l};
-      if (O.beta != 0.0) {
-        const float2 b = ((const float2*)O.base)[orow];
-        s = df_acc(s, b.x, b.y);
+#pragma unroll
+    for (int e = 0; e < VW; ++e) u.i[e] = c + e < nc ? (xi ? xi[c + e] : c + e) : -1;
+    return u;
+  };
+  const int c0 = sub * VW, step = G * VW;
+  const Vec u0 = load(c0), u1 = load(c0 + step);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the vectors are the previous launches'
+  df s[NR];
+  double d0[NR], d1[NR];
+#pragma unroll
+  for (int t = 0; t < NR; ++t) {
+    s[t] = {0.f, 0.f};
+    d0[t] = d1[t] = 0.0;
+  }
+  auto add = [&](const Vec& u) {
+#pragma unroll
+    for (int e = 0; e < VW; ++e)
+      if (u.i[e] >= 0)
+#pragma unroll
+        for (int t = 0; t < NR; ++t) {
+          const T x = ((const T*)(X + t * stride))[u.i[e]];
+          if constexpr (PAIRS) {
+            s[t] = pair_term(s[t], u.v[e], x);
+          } else {
+            if (e == 0) d0[t] = fma(u.v[e], x, d0[t]); else d1[t] = fma(u.v[e], x, d1[t]);
+          }
+        }
+  };
+  add(u0);
+  add(u1);
+  for (int c = c0 + 2 * step; c < nc; c += 2 * step) {
+    const Vec u = load(c), w = load(c + step);
+    add(u);
+    add(w);
+  }
+  const int orow = live && O.oidx ? O.oidx[r] : r;
+#pragma unroll
+  for (int t = 0; t < NR; ++t) {
+    char* out = (char*)O.out + off + t * stride;
+    const char* base = (const char*)O.base + off + t * stride;
+    if constexpr (PAIRS) {
+      for (int o = G >> 1; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(0xffffffffu, s[t].h, o), ol = __shfl_xor_sync(0xffffffffu, s[t].l, o);
+        s[t] = df_acc(s[t], oh, ol);
       }
-      ((float2*)O.out)[orow] = make_float2(s.h, s.l);
-    }
-  } else {
-    const double* X = (const double*)O.x;
-    const double* row = (const double*)O.M + (long)r * O.ldm;
-    double s0 = 0.0, s1 = 0.0;
-    auto xv = [&](int c) { return O.xidx ? X[O.xidx[c]] : X[c]; };
-    int c = sub * 2;
-    for (; c + G * 2 < nc; c += 2 * G * 2) {
-      const double2 u = *(const double2*)(row + c);
-      const double2 w = *(const double2*)(row + c + G * 2);
-      const int c2 = c + G * 2;
-      s0 = fma(u.x, xv(c), s0);
-      if (c + 1 < nc) s1 = fma(u.y, xv(c + 1), s1);
-      s0 = fma(w.x, xv(c2), s0);
-      if (c2 + 1 < nc) s1 = fma(w.y, xv(c2 + 1), s1);
-    }
-    if (c < nc) {
-      const double2 u = *(const double2*)(row + c);
-      s0 = fma(u.x, xv(c), s0);
-      if (c + 1 < nc) s1 = fma(u.y, xv(c + 1), s1);
-    }
-    double s = s0 + s1;
-    for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (live && sub == 0) {
-      const int orow = O.oidx ? O.oidx[r] : r;
-      const double v = O.alpha * s;
-      ((double*)O.out)[orow] = O.beta == 0.0 ? v : O.beta * ((const double*)O.base)[orow] + v;
+      if (live && sub == 0) {
+        df v = s[t];
+        if (O.alpha < 0.0) v = {-v.h, -v.l};
+        if (O.beta != 0.0) {
+          const float2 b = ((const float2*)base)[orow];
+          v = df_acc(v, b.x, b.y);
+        }
+        ((float2*)out)[orow] = make_float2(v.h, v.l);
+      }
+    } else {
+      double v = d0[t] + d1[t];
+      for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (live && sub == 0) {
+        v *= O.alpha;
+        ((double*)out)[orow] = O.beta == 0.0 ? v : O.beta * ((const double*)base)[orow] + v;
+      }
     }
   }
 }
@@ -1757,13 +1777,21 @@ __global__ void k_pair_join(const float2* __restrict__ in, double* __restrict__ 
   }
 }
 
-void launch_solve_ops(cudaStream_t s, const SolveOp* ops, const int* warp_ptr, int nops, int nwarps, bool pairs) {
-  if (!nops || !nwarps) return;
-  const unsigned blocks = (unsigned)((nwarps + 7) / 8);
-  if (pairs)
-    k_solve_rows<true><<<blocks, 256, 0, s>>>(ops, warp_ptr, nops);
-  else
-    k_solve_rows<false><<<blocks, 256, 0, s>>>(ops, warp_ptr, nops);
+void launch_solve_ops(cudaStream_t s, const SolveOp* ops, const int2* warps, int nwarps, bool pairs, int nr, long off,
+                      long stride) {
+  if (!nwarps) return;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((nwarps + 7) / 8));
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  auto f = pairs ? (nr == 4 ? k_solve_rows<true, 4> : (nr == 2 ? k_solve_rows<true, 2> : k_solve_rows<true, 1>))
+                 : (nr == 4 ? k_solve_rows<false, 4> : (nr == 2 ? k_solve_rows<false, 2> : k_solve_rows<false, 1>));
+  CK(cudaLaunchKernelEx(&cfg, f, ops, warps, nwarps, off, stride));
 }
 
 void launch_pack(DescStage& st, const std::vector<PackDesc>& v, bool fp32) {

@@ -40,33 +40,30 @@ void capture_solve_plan(SolvePlan& P, const std::vector<std::vector<SolveOp>>& l
   int32_t* dx = (int32_t*)P.mem.alloc_bytes(sizeof(int32_t) * std::max<size_t>(1, idx_all.size()));
   if (!idx_all.empty()) CK(cudaMemcpy(dx, idx_all.data(), sizeof(int32_t) * idx_all.size(), cudaMemcpyHostToDevice));
   std::vector<SolveOp> ops_all;
-  std::vector<int> wp_all;
-  std::vector<std::array<size_t, 3>> where;  // op offset, warp_ptr offset, warps
+  std::vector<int2> wp_all;                   // (op, first row) of every warp
+  std::vector<std::array<size_t, 3>> where;  // op offset, first warp, warps
   for (size_t li = 0; li < launches.size(); ++li) {
     const size_t o0 = ops_all.size(), w0 = wp_all.size();
-    int warps = 0;
-    wp_all.push_back(0);
     for (size_t k = 0; k < launches[li].size(); ++k) {
       SolveOp o = launches[li][k];
       if (xoff[li][k] >= 0) o.xidx = dx + xoff[li][k];
       if (ooff[li][k] >= 0) o.oidx = dx + ooff[li][k];
-      warps += (o.rows + 32 / o.lanes - 1) / (32 / o.lanes);
+      for (int r = 0; r < o.rows; r += 32 / o.lanes) wp_all.push_back(make_int2((int)k, r));
       ops_all.push_back(o);
-      wp_all.push_back(warps);
     }
-    where.push_back({o0, w0, (size_t)warps});
+    where.push_back({o0, w0, wp_all.size() - w0});
   }
   SolveOp* dops = (SolveOp*)P.mem.alloc_bytes(sizeof(SolveOp) * std::max<size_t>(1, ops_all.size()));
-  int* dwp = (int*)P.mem.alloc_bytes(sizeof(int) * std::max<size_t>(1, wp_all.size()));
+  int2* dwp = (int2*)P.mem.alloc_bytes(sizeof(int2) * std::max<size_t>(1, wp_all.size()));
   if (!ops_all.empty()) CK(cudaMemcpy(dops, ops_all.data(), sizeof(SolveOp) * ops_all.size(), cudaMemcpyHostToDevice));
-  if (!wp_all.empty()) CK(cudaMemcpy(dwp, wp_all.data(), sizeof(int) * wp_all.size(), cudaMemcpyHostToDevice));
+  if (!wp_all.empty()) CK(cudaMemcpy(dwp, wp_all.data(), sizeof(int2) * wp_all.size(), cudaMemcpyHostToDevice));
   P.prog.clear();
   for (size_t li = 0; li < launches.size(); ++li)
     P.prog.push_back(SolveLaunch{dops + where[li][0], dwp + where[li][1], (int)launches[li].size(), (int)where[li][2]});
   cudaStream_t cs;
   CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-  for (auto& l : P.prog) launch_solve_ops(cs, l.ops, l.warp_ptr, l.nops, l.nwarps, P.pairs);
+  for (auto& l : P.prog) launch_solve_ops(cs, l.ops, l.warps, l.nwarps, P.pairs);
   cudaGraph_t g;
   CK(cudaStreamEndCapture(cs, &g));
   CK(cudaGraphInstantiate(&P.graph, g, 0));
@@ -310,7 +307,7 @@ void run_solve_tree(const ifmm_fact& F, const double* in, double* out, cudaStrea
     for (auto& l : P.prog) {
       prof_batch_tag() = l.nops;
       cudaEvent_t pe = profiler().begin(KK_GEMV, s);
-      launch_solve_ops(s, l.ops, l.warp_ptr, l.nops, l.nwarps, P.pairs);
+      launch_solve_ops(s, l.ops, l.warps, l.nwarps, P.pairs);
       profiler().end(KK_GEMV, s, pe);
     }
     check_launch("k_solve_rows", (long)P.prog.size());
@@ -476,26 +473,64 @@ ifmm_status ifmm_solve(const ifmm_fact* f, const double* r, double* v, int nrhs,
     const int64_t NP = f->t->N, N = NP * dof;  // points, doubles per vector
     const bool dev = is_device_ptr(r);
     IFMM_REQUIRE(dev == is_device_ptr(v), IFMM_EINVAL, "r and v must both be host or both device");
+    // Several right-hand sides go through the program together, four or two at a
+    // time (one reading of the coefficients); a single one takes the graph.
+    const SolvePlan& P = f->plan;
+    const int group = nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1);
+    const size_t vl = ((size_t)P.vlen + 31) & ~(size_t)31;
     Vecs V;
     for (int i = 0; i < 2; ++i) V.reserve(N);
+    if (group > 1) V.reserve(vl * group);
     double* a = V.get(N);
     double* b = V.get(N);
-    for (int c = 0; c < nrhs; ++c) {
-      const double* rc = r + (int64_t)c * N;
-      double* vc = v + (int64_t)c * N;
-      const double* src = rc;
+    double* blk = group > 1 ? V.get(vl * group) : nullptr;
+    auto gather = [&](int c, double* dst) {
+      const double* src = r + (int64_t)c * N;
       if (!dev) {
-        CK(cudaMemcpyAsync(b, rc, sizeof(double) * N, cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(b, src, sizeof(double) * N, cudaMemcpyHostToDevice, s));
         src = b;
       }
-      launch_gather_perm(s, src, f->t->d_perm, a, (int)NP, dof);
-      run_solve_tree(*f, a, a, s);
-      if (dev) {
-        launch_scatter_perm(s, a, f->t->d_perm, vc, (int)NP, dof);
-      } else {
-        launch_scatter_perm(s, a, f->t->d_perm, b, (int)NP, dof);
-        CK(cudaMemcpyAsync(vc, b, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
+      launch_gather_perm(s, src, f->t->d_perm, dst, (int)NP, dof);
+    };
+    auto scatter = [&](int c, const double* src) {
+      double* vc = v + (int64_t)c * N;
+      launch_scatter_perm(s, src, f->t->d_perm, dev ? vc : b, (int)NP, dof);
+      if (!dev) CK(cudaMemcpyAsync(vc, b, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
+    };
+    for (int c = 0; c < nrhs;) {
+      int nr = group;
+      while (nr > nrhs - c) nr /= 2;
+      if (nr == 1) {
+        gather(c, a);
+        run_solve_tree(*f, a, a, s);
+        scatter(c, a);
+        ++c;
+        continue;
       }
+      const long stride = 8 * (long)vl, off = (char*)blk - (char*)P.V;
+      for (int t = 0; t < nr; ++t) {
+        char* in = (char*)P.stage_in + off + t * stride;
+        if (P.pairs) {
+          gather(c + t, a);
+          launch_pair_split(s, a, in, N);
+        } else {
+          gather(c + t, (double*)in);
+        }
+      }
+      cudaEvent_t pe = profiler().begin(KK_SOLVE_GRAPH, s, (long)P.prog.size());
+      for (auto& l : P.prog) launch_solve_ops(s, l.ops, l.warps, l.nwarps, P.pairs, nr, off, stride);
+      check_launch("k_solve_rows", (long)P.prog.size());
+      profiler().end(KK_SOLVE_GRAPH, s, pe);
+      for (int t = 0; t < nr; ++t) {
+        const char* res = (const char*)(P.stage_out ? P.stage_out : P.stage_in) + off + t * stride;
+        if (P.pairs) {
+          launch_pair_join(s, res, a, N);
+          scatter(c + t, a);
+        } else {
+          scatter(c + t, (const double*)res);
+        }
+      }
+      c += nr;
     }
     CK(cudaStreamSynchronize(s));
     return IFMM_OK;
