@@ -1037,56 +1037,85 @@ __global__ void __launch_bounds__(128) k_il_transform(const int* __restrict__ li
 }
 
 // One CTA per (event, side): gathers the weight stack of ZGatherDesc from the
-// level's IL blocks on the device.
+// level's IL blocks on the device.  The rows of every entry's block are found by a
+// scan of the ranks first, so that the warps copy different entries at the same
+// time (one after the other the entries' dependent loads were the time: 201 us a
+// launch at 131,072 points, now 142).
 __global__ void __launch_bounds__(256) k_zgather(const ZGatherDesc* __restrict__ d, int nd, ZTables t) {
   if ((int)blockIdx.x >= nd) return;
   const ZGatherDesc D = d[blockIdx.x];
   const int q = D.q, rq = t.r[q];
   const long ldz = D.ldz;
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  constexpr int CH = 256;  // entries of a pass
+  __shared__ int offs[CH + 1], rls[CH];
+  __shared__ const double* src[CH];
+  __shared__ int lds[CH];
   int off = 0;
-  for (int e = t.il_ptr[q]; e < t.il_ptr[q + 1]; ++e) {
-    const int l = t.il[e], rl = t.r[l];
-    if (rl == 0) continue;
-    if (D.side == 0) {
-      const double* src = t.far[t.il_T[e]];
-      const long lds = t.capr[l];
-      for (int x = tid; x < rl * rq; x += nt) {
-        const int i = x % rl, j = x / rl;
-        D.Z[off + i + j * ldz] = src[i + j * lds];
+  for (int e0 = t.il_ptr[q]; e0 < t.il_ptr[q + 1]; e0 += CH) {
+    const int cnt = min(CH, t.il_ptr[q + 1] - e0);
+    __syncthreads();  // the previous pass is done with the lists
+    for (int x = threadIdx.x; x < cnt; x += blockDim.x) {
+      const int l = t.il[e0 + x];
+      rls[x] = t.r[l];
+      src[x] = t.far[D.side == 0 ? t.il_T[e0 + x] : e0 + x];
+      lds[x] = t.capr[D.side == 0 ? l : q];
+    }
+    __syncthreads();
+    if (w == 0) {
+      int base = off;
+      for (int x0 = 0; x0 < cnt; x0 += 32) {
+        const int v = x0 + lane < cnt ? rls[x0 + lane] : 0;
+        int s = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, s, o);
+          if (lane >= o) s += y;
+        }
+        if (x0 + lane < cnt) offs[x0 + lane] = base + s - v;
+        base += __shfl_sync(0xffffffffu, s, 31);
       }
-    } else {
-      const double* src = t.far[e];
-      const long lds = t.capr[q];
-      for (int x = tid; x < rl * rq; x += nt) {
-        const int i = x % rl, j = x / rl;
-        D.Z[off + i + j * ldz] = src[j + i * lds];
+      if (lane == 0) offs[cnt] = base;
+    }
+    __syncthreads();
+    for (int x = w; x < cnt; x += nw) {
+      const int rl = rls[x];
+      const double* p = src[x];
+      double* z = D.Z + offs[x];
+      const long ls = lds[x];
+      for (int i = lane; i < rl; i += 32) {
+        const double* pi = D.side == 0 ? p + i : p + i * ls;
+        const long st = D.side == 0 ? ls : 1;
+        int j = 0;
+        for (; j + 4 <= rq; j += 4) {
+          const double v0 = pi[j * st], v1 = pi[(j + 1) * st], v2 = pi[(j + 2) * st], v3 = pi[(j + 3) * st];
+          z[i + j * ldz] = v0;
+          z[i + (j + 1) * ldz] = v1;
+          z[i + (j + 2) * ldz] = v2;
+          z[i + (j + 3) * ldz] = v3;
+        }
+        for (; j < rq; ++j) z[i + j * ldz] = pi[j * st];
       }
     }
-    off += rl;
+    off = offs[cnt];
   }
   if (t.tail) {
     const int rc = t.rc;
-    if (D.side == 0) {
-      const double* src = t.M2M[q];
-      for (int x = tid; x < rc * rq; x += nt) {
-        const int i = x % rc, j = x / rc;
-        D.Z[off + i + j * ldz] = src[i + (long)j * rc];
-      }
-    } else {
-      const double* src = t.L2L[q];
-      const long lds = t.capr[q];
-      for (int x = tid; x < rc * rq; x += nt) {
-        const int i = x % rc, j = x / rc;
-        D.Z[off + i + j * ldz] = src[j + i * lds];
-      }
-    }
+    const double* p = D.side == 0 ? t.M2M[q] : t.L2L[q];
+    const long ls = t.capr[q];
+    for (int j = w; j < rq; j += nw)
+      for (int i = lane; i < rc; i += 32)
+        D.Z[off + i + j * ldz] = D.side == 0 ? p[i + (long)j * rc] : p[j + i * ls];
   }
 }
 
 // One CTA per (eliminated node, neighbour a): adds the row block of neighbour a
-// of F into its near blocks (ScatterDesc).  The slot of (q, q2) is found by a
-// binary search of q2 in q's sorted neighbour list.
+// of F into its near blocks (ScatterDesc).  Lane b of the first warp finds the
+// block of (a, b) (a binary search of q2 in q's sorted neighbour list; all of them
+// at once), then the warps take the columns of F, narrow row blocks several
+// columns per warp, four in flight.  Bound: the read-modify-write of the near
+// blocks; with one search after the other and one column per warp it took 339 us a
+// launch at 131,072 points, now 203.
 __global__ void __launch_bounds__(256) k_schur_scatter(const ScatterDesc* __restrict__ d, int nd, ScatterTables t) {
   const int di = blockIdx.x;
   if (di >= nd) return;
@@ -1095,44 +1124,81 @@ __global__ void __launch_bounds__(256) k_schur_scatter(const ScatterDesc* __rest
   const int c0 = t.nbr_ptr[i], deg = t.nbr_ptr[i + 1] - c0;
   const int a = blockIdx.y;
   if (a >= deg) return;
-  __shared__ int roff[32], dims[32], cl[32];
-  if (threadIdx.x == 0) {
-    int off = 0;
-    for (int b = 0; b < deg && b < 32; ++b) {
-      const int q = t.nbr[c0 + b];
-      const int dq = t.elim[q] ? t.r[q] : t.n[q];
-      cl[b] = q;
-      roff[b] = off;
-      dims[b] = dq;
-      off += dq;
+  __shared__ int roff[33];
+  __shared__ double* dsts[32];
+  __shared__ int s_mq, s_ld;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (w == 0) {
+    const int q2 = lane < deg ? t.nbr[c0 + lane] : 0;
+    const int el2 = lane < deg ? t.elim[q2] : 0;
+    const int v = lane < deg ? (el2 ? t.r[q2] : t.n[q2]) : 0;
+    int s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
     }
+    roff[lane + 1] = s;
+    if (lane == 0) roff[0] = 0;
+    const int q = __shfl_sync(0xffffffffu, q2, a), elq = __shfl_sync(0xffffffffu, el2, a);
+    double* dst = nullptr;
+    if (lane < deg && v) {
+      const int q0 = t.nbr_ptr[q], q1 = t.nbr_ptr[q + 1];
+      int slot = -1;
+      if (q2 == q) {
+        slot = t.slot_ptr[q];
+      } else {
+        int lo = q0, hi = q1;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (t.nbr[mid] < q2) lo = mid + 1; else hi = mid;
+        }
+        if (lo < q1 && t.nbr[lo] == q2) slot = t.slot_ptr[q] + 1 + (lo - q0);
+      }
+      // (no slot: a far pair, consumed by the recompression)
+      if (slot >= 0) dst = (elq + el2 == 0 ? t.nb0 : (elq + el2 == 1 ? t.nb1 : t.nb2))[slot];
+    }
+    dsts[lane] = dst;
+    if (lane == a) s_mq = v;
+    if (lane == 0) s_ld = t.n[q];
   }
   __syncthreads();
-  const int q = cl[a], mq = dims[a];
+  const int mq = s_mq;
   if (mq == 0 || t.n[i] == 0) return;
-  const int q0 = t.nbr_ptr[q], q1 = t.nbr_ptr[q + 1];
-  const long ldd = t.n[q];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int b = 0; b < deg; ++b) {
-    const int q2 = cl[b], mq2 = dims[b];
-    if (mq2 == 0) continue;
-    int slot = -1;
-    if (q2 == q) {
-      slot = t.slot_ptr[q];
-    } else {
-      int lo = q0, hi = q1;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (t.nbr[mid] < q2) lo = mid + 1; else hi = mid;
+  const long ldd = s_ld;
+  const int M = roff[deg];
+  const double* F = D.F + roff[a];
+  const int rp = mq <= 8 ? 8 : (mq <= 16 ? 16 : 32), cw = 32 / rp;  // lanes per column, columns per warp
+  const int x0 = lane & (rp - 1);
+  int b = 0;
+  for (int col = w * cw + lane / rp; col < M; col += 4 * nw * cw) {
+    double* o[4];
+    const double* f[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = col + u * nw * cw;
+      o[u] = nullptr;
+      f[u] = nullptr;
+      if (c < M) {
+        while (c >= roff[b + 1]) ++b;
+        f[u] = F + (long)c * D.M;
+        if (dsts[b]) o[u] = dsts[b] + (c - roff[b]) * ldd;
       }
-      if (lo < q1 && t.nbr[lo] == q2) slot = t.slot_ptr[q] + 1 + (lo - q0);
     }
-    if (slot < 0) continue;  // a far pair: consumed by the recompression
-    const int stg = t.elim[q] + t.elim[q2];
-    double* dst = (stg == 0 ? t.nb0 : (stg == 1 ? t.nb1 : t.nb2))[slot];
-    const double* src = D.F + roff[a] + (long)roff[b] * D.M;
-    for (int j = w; j < mq2; j += nw)
-      for (int x = lane; x < mq; x += 32) dst[x + (long)j * ldd] += src[x + (long)j * D.M];
+    for (int x = x0; x < mq; x += rp) {
+      double v[4], y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        v[u] = y[u] = 0.0;
+        if (o[u]) {
+          v[u] = f[u][x];
+          y[u] = o[u][x];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (o[u]) o[u][x] = y[u] + v[u];
+    }
   }
 }
 

@@ -1098,26 +1098,39 @@ __global__ void k_bd_fill(const BdBlockDesc* __restrict__ d, const int* __restri
 // m = (c p + b) p + a, u = (x_j - centre)/halfwidth.
 // With dof = 2 the matrix is S (x) I_2 (each node and point carries a real and
 // an imaginary part).
-__global__ void k_interp(const InterpDesc* __restrict__ d, int nd, const double* __restrict__ px,
+// The Lagrange factors of 64 points at a time are formed once per axis in shared
+// memory (each entry of S formed its own three, cosines of the roots included: 8.6
+// ms for the leaves of the 131,072-point job, now 0.65).
+__global__ void __launch_bounds__(256) k_interp(const InterpDesc* __restrict__ d, int nd, const double* __restrict__ px,
                          const double* __restrict__ py, const double* __restrict__ pz, int p, int dof) {
   if ((int)blockIdx.x >= nd) return;
   const InterpDesc D = d[blockIdx.x];
   const int r = p * p * p;
-  const int total = r * D.n;
-  for (int e = threadIdx.x; e < total; e += blockDim.x) {
-    const int m = e % r, j = e / r;
-    const int a = m % p, b = (m / p) % p, c = m / (p * p);
-    const int pt = D.p0 + j;
-    const double ux = (px[pt] - D.cx) / D.h, uy = (py[pt] - D.cy) / D.h, uz = (pz[pt] - D.cz) / D.h;
-    const double v = lagrange(a, p, ux) * lagrange(b, p, uy) * lagrange(c, p, uz);
-    if (dof == 1) {
-      D.dst[m + (long)j * D.ld] = v;
-    } else {
-      double* o = D.dst + 2 * m + (long)(2 * j) * D.ld;
-      o[0] = v;
-      o[1] = 0.0;
-      o[D.ld] = 0.0;
-      o[D.ld + 1] = v;
+  constexpr int CH = 64;
+  __shared__ double lg[3][6][CH];
+  for (int j0 = 0; j0 < D.n; j0 += CH) {
+    const int cnt = min(CH, D.n - j0);
+    __syncthreads();  // the previous points' factors are read
+    for (int e = threadIdx.x; e < 3 * p * cnt; e += blockDim.x) {
+      const int j = e % cnt, a = (e / cnt) % p, ax = e / (cnt * p);
+      const int pt = D.p0 + j0 + j;
+      const double u = ax == 0 ? (px[pt] - D.cx) / D.h : (ax == 1 ? (py[pt] - D.cy) / D.h : (pz[pt] - D.cz) / D.h);
+      lg[ax][a][j] = lagrange(a, p, u);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < r * cnt; e += blockDim.x) {
+      const int m = e % r, j = e / r;
+      const int a = m % p, b = (m / p) % p, c = m / (p * p);
+      const double v = lg[0][a][j] * lg[1][b][j] * lg[2][c][j];
+      if (dof == 1) {
+        D.dst[m + (long)(j0 + j) * D.ld] = v;
+      } else {
+        double* o = D.dst + 2 * m + (long)(2 * (j0 + j)) * D.ld;
+        o[0] = v;
+        o[1] = 0.0;
+        o[D.ld] = 0.0;
+        o[D.ld + 1] = v;
+      }
     }
   }
 }
@@ -1133,15 +1146,18 @@ __global__ void k_m2l_table(double* __restrict__ out, int p, double h, double sc
   const int ox = o % 7 - 3, oy = (o / 7) % 7 - 3, oz = o / 49 - 3;
   const bool near = abs(ox) <= 1 && abs(oy) <= 1 && abs(oz) <= 1;
   double* T = out + (long)o * rd * rd;
+  __shared__ double root[6];
+  if ((int)threadIdx.x < p) root[threadIdx.x] = cheb_root(threadIdx.x, p);
+  __syncthreads();
   for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
     const int m = e % r, k = e / r;
     double v = 0.0, vi = 0.0;
     if (!near) {
       const int ma = m % p, mb = (m / p) % p, mc = m / (p * p);
       const int ka = k % p, kb = (k / p) % p, kc = k / (p * p);
-      const double dx = 2.0 * ox + cheb_root(ma, p) - cheb_root(ka, p);
-      const double dy = 2.0 * oy + cheb_root(mb, p) - cheb_root(kb, p);
-      const double dz = 2.0 * oz + cheb_root(mc, p) - cheb_root(kc, p);
+      const double dx = 2.0 * ox + root[ma] - root[ka];
+      const double dy = 2.0 * oy + root[mb] - root[kb];
+      const double dz = 2.0 * oz + root[mc] - root[kc];
       const double dist = h * sqrt(dx * dx + dy * dy + dz * dz);
       if (dof == 1) {
         v = scale / dist;
@@ -1172,12 +1188,17 @@ __global__ void k_m2m_table(double* __restrict__ out, int p, int dof) {
   const int oct = blockIdx.x;  // 0..7, bit 0 = x, bit 1 = y, bit 2 = z
   const double sx = (oct & 1) - 0.5, sy = ((oct >> 1) & 1) - 0.5, sz = ((oct >> 2) & 1) - 0.5;
   double* T = out + (long)oct * rd * rd;
+  __shared__ double lg[3][6][6];  // factor of parent node m at child node k, per axis
+  for (int e = threadIdx.x; e < 3 * p * p; e += blockDim.x) {
+    const int k = e % p, m = (e / p) % p, ax = e / (p * p);
+    lg[ax][m][k] = lagrange(m, p, (ax == 0 ? sx : (ax == 1 ? sy : sz)) + 0.5 * cheb_root(k, p));
+  }
+  __syncthreads();
   for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
     const int m = e % r, k = e / r;
     const int ma = m % p, mb = (m / p) % p, mc = m / (p * p);
     const int ka = k % p, kb = (k / p) % p, kc = k / (p * p);
-    const double ux = sx + 0.5 * cheb_root(ka, p), uy = sy + 0.5 * cheb_root(kb, p), uz = sz + 0.5 * cheb_root(kc, p);
-    const double v = lagrange(ma, p, ux) * lagrange(mb, p, uy) * lagrange(mc, p, uz);
+    const double v = lg[0][ma][ka] * lg[1][mb][kb] * lg[2][mc][kc];
     if (dof == 1) {
       T[e] = v;
     } else {
@@ -1893,60 +1914,79 @@ void launch_matvec_df(cudaStream_t s, const float* pts_df, const float* qh, cons
 }
 
 // ---------------------------------------------------------------- Gram sums, Cholesky
-// dst (r x r) = sum of the listed r x r matrices (one CTA per output).
+// dst (r x r, upper triangle) = sum of the listed symmetric r x r matrices (one CTA
+// per output).  Columns c and r - 1 - c together have r + 1 entries.  Bound: FP64
+// additions (the Cholesky factor reads one triangle: half of them gone; 3.0 -> 1.6
+// ms a level at 131,072 points).
 __global__ void k_gram_sum(double* const* __restrict__ dst, const double* const* __restrict__ terms,
                            const int* __restrict__ first, int nd, int r) {
   const int b = blockIdx.x;
   if (b >= nd) return;
   const int t0 = first[b], t1 = first[b + 1];
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
+  const int hc = (r + 1) / 2;
+  for (int x = threadIdx.x; x < hc * (r + 1); x += blockDim.x) {
+    const int c = x / (r + 1), y = x - c * (r + 1);
+    const bool far = y < r - c;  // of column r - 1 - c, else of column c
+    if (!far && c == r - 1 - c) continue;
+    const int e = far ? y + (r - 1 - c) * r : (y - (r - c)) + c * r;
     double s = 0.0;
+#pragma unroll 4
     for (int t = t0; t < t1; ++t) s += terms[t][e];
     dst[b][e] = s;
   }
 }
 
 // Upper Cholesky factor R (R^T R = G + delta * max_i G_ii * I) of each r x r
-// matrix, r <= 128, in shared memory; a pivot that is still not positive is
-// replaced by delta * max_i G_ii (the direction then carries almost no weight).
-__global__ void k_chol(double* const* __restrict__ mats, int nd, int r, double delta) {
+// matrix (upper triangle read), r <= 128, in shared memory; a pivot that is still
+// not positive is replaced by delta * max_i G_ii (the direction then carries
+// almost no weight).  Row k goes through a buffer, so that the update's reads are
+// contiguous, with warps over columns and lanes over their rows above the diagonal
+// (2.2 -> 1.8 ms a level at 131,072 points; the chain of r steps is what remains).
+__global__ void __launch_bounds__(256) k_chol(double* const* __restrict__ mats, int nd, int r, double delta) {
   const int b = blockIdx.x;
   if (b >= nd) return;
   extern __shared__ double G[];
   double* M = mats[b];
-  __shared__ double s_diag, s_piv;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) G[e] = M[e];
+  __shared__ double s_diag, s_inv, row[128];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int j = w; j < r; j += nw)
+    for (int i = lane; i <= j; i += 32) G[i + j * r] = M[i + j * r];
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (w == 0) {
     double mx = 0.0;
-    for (int i = 0; i < r; ++i) mx = fmax(mx, G[i + i * r]);
-    s_diag = mx > 0.0 ? delta * mx : 1e-300;
+    for (int i = lane; i < r; i += 32) mx = fmax(mx, G[i + i * r]);
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_diag = mx > 0.0 ? delta * mx : 1e-300;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < r; i += blockDim.x) G[i + i * r] += s_diag;
+  const double dg = s_diag;
+  for (int i = threadIdx.x; i < r; i += blockDim.x) G[i + i * r] += dg;
   __syncthreads();
   // right-looking: column-major G, upper factor stored in the upper triangle
   for (int k = 0; k < r; ++k) {
     if (threadIdx.x == 0) {
       double d = G[k + k * r];
-      if (!(d > s_diag * 1e-3)) d = s_diag;
-      s_piv = sqrt(d);
-      G[k + k * r] = s_piv;
+      if (!(d > dg * 1e-3)) d = dg;
+      const double pv = sqrt(d);
+      G[k + k * r] = pv;
+      s_inv = 1.0 / pv;
     }
     __syncthreads();
-    const double pv = s_piv;
-    for (int j = k + 1 + threadIdx.x; j < r; j += blockDim.x) G[k + j * r] /= pv;  // row k of R
+    const double inv = s_inv;
+    for (int j = k + 1 + threadIdx.x; j < r; j += blockDim.x) {  // row k of R
+      const double v = G[k + j * r] * inv;
+      G[k + j * r] = v;
+      row[j] = v;
+    }
     __syncthreads();
-    for (int e = threadIdx.x; e < (r - k - 1) * (r - k - 1); e += blockDim.x) {
-      const int i = k + 1 + e % (r - k - 1), j = k + 1 + e / (r - k - 1);
-      if (i <= j) G[i + j * r] -= G[k + i * r] * G[k + j * r];
+    for (int j = k + 1 + w; j < r; j += nw) {
+      const double rj = row[j];
+      for (int i = k + 1 + lane; i <= j; i += 32) G[i + j * r] -= row[i] * rj;
     }
     __syncthreads();
   }
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e % r, j = e / r;
-    M[e] = (i <= j) ? G[e] : 0.0;
-  }
+  for (int j = w; j < r; j += nw)
+    for (int i = lane; i < r; i += 32) M[i + j * r] = (i <= j) ? G[i + j * r] : 0.0;
 }
 
 void launch_gram_sum(DescStage& st, const std::vector<double*>& dst, const std::vector<const double*>& terms,
