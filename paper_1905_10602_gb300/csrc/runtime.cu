@@ -759,26 +759,44 @@ void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
   }
 }
 
-template <typename TC>
-static void svd_rt_launch(int c, const SvdRtDesc* d, unsigned g, int threads, int slot, cudaStream_t s) {
-  static std::once_flag attr_once;
+template <typename TC, int G, int EM>
+static void svd_rt_run(const SvdRtDesc* d, unsigned g, int R, int threads, int slot, cudaStream_t s) {
   static constexpr int cap = 220 * 1024;
+  static std::once_flag attr_once;
   std::call_once(attr_once, [] {
-    CK(cudaFuncSetAttribute(k_svd_rt<TC, 8, 6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    CK(cudaFuncSetAttribute(k_svd_rt<TC, 16, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    CK(cudaFuncSetAttribute(k_svd_rt<TC, 32, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    CK(cudaFuncSetAttribute(k_svd_rt<TC, 32, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    CK(cudaFuncSetAttribute(k_svd_rt<TC, G, EM, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    if constexpr (sizeof(TC) == 8)
+      CK(cudaFuncSetAttribute(k_svd_rt<TC, G, EM, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   });
+  if (R == 1 || sizeof(TC) == 4) {
+    k_svd_rt<TC, G, EM, false, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+    return;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g * (unsigned)R);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)slot;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)R;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if constexpr (sizeof(TC) == 8) CK(cudaLaunchKernelEx(&cfg, k_svd_rt<TC, G, EM, false, true>, d, (int)g, 60, slot));
+}
+template <typename TC>
+static void svd_rt_launch(int c, const SvdRtDesc* d, unsigned g, int R, int threads, int slot, cudaStream_t s) {
   if (c == 0)
-    k_svd_rt<TC, 4, 4, true><<<(g + 3) / 4, 128, 4 * slot, s>>>(d, (int)g, 60, slot);
+    k_svd_rt<TC, 4, 4, true, false><<<(g + 3) / 4, 128, 4 * slot, s>>>(d, (int)g, 60, slot);
   else if (c == 1)
-    k_svd_rt<TC, 8, 6, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+    svd_rt_run<TC, 8, 6>(d, g, R, threads, slot, s);
   else if (c == 2)
-    k_svd_rt<TC, 16, 8, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+    svd_rt_run<TC, 16, 8>(d, g, R, threads, slot, s);
   else if (c == 3)
-    k_svd_rt<TC, 32, 8, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+    svd_rt_run<TC, 32, 8>(d, g, R, threads, slot, s);
   else
-    k_svd_rt<TC, 32, 0, false><<<g, threads, slot, s>>>(d, (int)g, 60, slot);
+    svd_rt_run<TC, 32, 0>(d, g, R, threads, slot, s);
   check_launch("k_svd_rt");
 }
 
@@ -823,17 +841,25 @@ void launch_svd_rt(DescStage& st, const std::vector<SvdRtDesc>& v, int prec) {
   for (int c = 4; c >= 0; --c) {  // the longest first
     if (part[c].empty()) continue;
     const size_t tail = svd_tail_bytes(nmx[c], tcb);
-    const int slot = (int)std::min<size_t>(
-        smem_cap, ((size_t)svd_ld(nmx[c], grp[c]) * nmx[c] * tcb + tail + 15) & ~(size_t)15);
+    auto slot_of = [&](int cols) { return ((size_t)svd_ld(nmx[c], grp[c]) * cols * tcb + tail + 15) & ~(size_t)15; };
     const unsigned g = (unsigned)part[c].size();
     // lanes for every pair of a problem that keeps all (class 1) or about half
     // (wider) of its columns; more warps than that only wait at the rounds' barriers
     const int pairs = c == 1 ? (nmx[c] + 1) / 2 : (nmx[c] + 3) / 4;
-    const int threads = std::min(g < 152 ? 1024 : 512, std::max(64, (pairs * grp[c] + 31) / 32 * 32));
+    // FP64: a cluster per problem where the batch leaves SMs idle and every CTA has
+    // at least two warps of pairs (8,192-point job 733 -> 592 ms; with one warp or
+    // four 600).  FP32 is not bound by one SM's arithmetic: with clusters its jobs
+    // took 0 to 1 % longer (131,072 points 1024 -> 1027 to 1035 ms).
+    int R = 1;
+    for (int q = 2; q <= 8 && c > 0 && prec == P64; q *= 2)
+      if (g * (unsigned)q <= 152 && pairs * grp[c] >= 64 * q && slot_of((nmx[c] + q - 1) / q) <= smem_cap) R = q;
+    const int slot = (int)std::min(smem_cap, slot_of((nmx[c] + R - 1) / R));
+    const int lanes = (pairs + R - 1) / R * grp[c];
+    const int threads = std::min(g < 152 ? 1024 : 512, std::max(64, (lanes + 31) / 32 * 32));
     if (prec == P32)
-      svd_rt_launch<float>(c, d[c], g, threads, slot, fj.stream(li++));
+      svd_rt_launch<float>(c, d[c], g, R, threads, slot, fj.stream(li++));
     else
-      svd_rt_launch<double>(c, d[c], g, threads, slot, fj.stream(li++));
+      svd_rt_launch<double>(c, d[c], g, R, threads, slot, fj.stream(li++));
   }
   fj.join();
   profiler().end(kk, st.stream, pe);
