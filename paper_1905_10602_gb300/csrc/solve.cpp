@@ -452,6 +452,19 @@ struct Vecs {
   }
 };
 
+// One more block that a faster kernel wants and the call can do without: null when
+// the device has no room for it.
+static double* get_or_null(Vecs& W, size_t n) {
+  try {
+    W.total = 0;
+    W.reserve(n);
+    return W.get(n);
+  } catch (const Error& e) {
+    if (e.code != IFMM_ENOMEM) throw;
+    return nullptr;
+  }
+}
+
 // doubles of the partial-sum buffer of the symmetric float-pair matvec, when it
 // is at most 8 GiB (N up to about 300,000 points) and this tree may take that
 // kernel; 0 otherwise
@@ -476,14 +489,15 @@ ifmm_status ifmm_solve(const ifmm_fact* f, const double* r, double* v, int nrhs,
     // Several right-hand sides go through the program together, four or two at a
     // time (one reading of the coefficients); a single one takes the graph.
     const SolvePlan& P = f->plan;
-    const int group = nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1);
+    int group = nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1);
     const size_t vl = ((size_t)P.vlen + 31) & ~(size_t)31;
-    Vecs V;
+    Vecs V, W;
     for (int i = 0; i < 2; ++i) V.reserve(N);
-    if (group > 1) V.reserve(vl * group);
     double* a = V.get(N);
     double* b = V.get(N);
-    double* blk = group > 1 ? V.get(vl * group) : nullptr;
+    double* blk = nullptr;
+    // where a group's vectors do not fit: a smaller group, then one after the other
+    while (group > 1 && !(blk = get_or_null(W, vl * group))) group /= 2;
     auto gather = [&](int c, double* dst) {
       const double* src = r + (int64_t)c * N;
       if (!dev) {
@@ -557,9 +571,9 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
     const bool df_mv = k->arith == IFMM_ARITH_DF, fmm_mv = k->arith == IFMM_ARITH_FMM;
     // partial sums of the symmetric kernels
     const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
-    Vecs V;
+    Vecs V, W;
     for (int i = 0; i < (df_mv ? 4 : 3); ++i) V.reserve(N);
-    if (np) V.reserve(np);
+    if (df_mv && np) V.reserve(np);
     double* a = V.get(N);
     double* b = V.get(N);
     double* c = V.get(N);
@@ -580,7 +594,7 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
       const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, q, a, b, N, k, part);
       launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, part);
     } else {
-      launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? V.get(np) : nullptr);
+      launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? get_or_null(W, np) : nullptr);
     }
     if (dev) {
       launch_scatter_perm(s, b, t->d_perm, y, (int)NP, dof);
@@ -621,13 +635,13 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     // another kernel, or FP64)
     const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
     const size_t nkp = (size_t)kry_parts(N) * 2 * m;
-    Vecs Vm;
+    Vecs Vm, W;
     for (int i = 0; i < 6; ++i) Vm.reserve(N);
     Vm.reserve((size_t)N * (m + 1));
     Vm.reserve(2 * (size_t)m + 2);
     Vm.reserve(nkp);
     if (df_mv) Vm.reserve(N);
-    if (np) Vm.reserve(np);
+    if (df_mv && np) Vm.reserve(np);
     double* bt = Vm.get(N);   // b in tree order
     double* xt = Vm.get(N);   // x in tree order
     double* rt = Vm.get(N);
@@ -638,7 +652,7 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     double* kp = Vm.get(nkp);
     double* tmp = Vm.get(N);
     float* qdf = df_mv ? (float*)Vm.get(N) : nullptr;
-    double* part = np ? Vm.get(np) : nullptr;
+    double* part = !np ? nullptr : (df_mv ? Vm.get(np) : get_or_null(W, np));
     const double* src = b;
     if (!dev) {
       CK(cudaMemcpyAsync(tmp, b, sizeof(double) * N, cudaMemcpyHostToDevice, s));
