@@ -4,8 +4,8 @@
 //
 // Every matrix is column-major with a leading dimension (BLAS convention).
 // One descriptor describes one problem; a launch covers a batch of problems of
-// different sizes (the nodes of one color of one level).  Kernels never wait
-// on anything but __syncthreads, and every index is bounded by the sizes in
+// different sizes (the nodes of one color of one level).  Kernels wait only on
+// block and cluster barriers, and every index is bounded by the sizes in
 // the descriptor.
 #pragma once
 
