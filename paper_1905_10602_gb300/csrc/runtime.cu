@@ -423,7 +423,12 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
   while (qwant < 4 && (nbig << (qwant + 1)) <= kMul * 152) ++qwant;
   std::vector<InvDesc> cls[6][5], rest;
   size_t smx[6][5] = {};
+  size_t ncls = 0;
   for (auto& x : v) {
+    if (x.n < 1) {  // nothing to invert: the kernels' steps and barriers need a column
+      CK(cudaMemsetAsync(x.info, 0, sizeof(int), st.stream));
+      continue;
+    }
     int c = 0;
     while (c < 6 && x.n > kRows[c]) ++c;
     if ((fallback_n && x.n >= fallback_n) || c == 6) {
@@ -449,15 +454,16 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
       rest.push_back(x);
       continue;
     }
+    ++ncls;
     cls[c][q].push_back(x);
     smx[c][q] = std::max(smx[c][q], inv_slot_bytes(x.n, 1 << q));
   }
-  if (rest.size() < v.size()) {
+  if (ncls) {
     const InvDesc* dcl[6][5] = {};
     for (int c = 0; c < 6; ++c)
       for (int q = 0; q < 5; ++q)
         if (!cls[c][q].empty()) dcl[c][q] = st.push(cls[c][q]);
-    prof_batch_tag() = (long)(v.size() - rest.size());
+    prof_batch_tag() = (long)ncls;
     cudaEvent_t pe = profiler().begin(KK_INV, st.stream);
     ForkJoin fj(st.stream);
     int li = 0;
