@@ -648,26 +648,35 @@ static std::vector<size_t> launch_qr_reg(DescStage& st, const std::vector<QrcpDe
     // 256 rows even where they would fit as a whole: eight rows per lane leave
     // registers for three times as many problems per SM.  Measured (all QR of one
     // level): 131,072 points, level 5: 120 -> 71 ms, 8,192 points FP64, level 3:
-    // 124 -> 101; narrower blocks lose (level 6: 18 -> 36 ms).
-    const int tall = x.rb == 0 && x.n > kQrWarpCols && x.n <= 64 && x.m > 384 ? 256 : 0;
+    // 124 -> 101; narrower blocks lose (level 6: 18 -> 36 ms).  Where the stacked R
+    // factors of 256-row chunks have no plan (more than 256 * 1536 / n rows) the
+    // chunks are doubled until they have one (7,000 x 64 FP32: 21.7 ms in the global-memory
+    // kernel, 0.8 by chunks of 512).
+    const int cmax = 32 * kQrRows[kQrClasses - 1];
+    const bool tall = x.rb == 0 && x.n > kQrWarpCols && x.n <= 64 && x.m > 384;
     if (!tall && resident(qr_plan(x.m, x.n, tcb))) {
       fit.push_back(x);
       continue;
     }
-    // else the tallest chunk that has a plan (a multiple of 32 rows)
-    int c = tall ? tall : 32 * kQrRows[kQrClasses - 1];
-    while (c > x.n && !resident(qr_plan(c, x.n, tcb))) c -= 32;
-    if (x.rb > 0 || x.m <= x.n || c <= x.n) {
+    // rows of the stacked R factors of chunks of c rows
+    auto stacked = [&](int c) {
+      const int nch = (x.m + c - 1) / c;
+      return (nch - 1) * x.n + std::min(x.n, x.m - (nch - 1) * c);
+    };
+    auto reduces = [&](int c) {
+      return c > x.n && resident(qr_plan(c, x.n, tcb)) && resident(qr_plan(stacked(c), x.n, tcb));
+    };
+    int c = tall ? 256 : cmax;
+    while (tall && c < cmax && !reduces(c)) c = std::min(2 * c, cmax);
+    if (!reduces(c)) {  // the tallest chunk that has a plan (a multiple of 32 rows)
+      c = tall ? 256 : cmax;
+      while (c > x.n && !resident(qr_plan(c, x.n, tcb))) c -= 32;
+    }
+    if (x.rb > 0 || x.m <= x.n || !reduces(c)) {
       rest.push_back(i);
       continue;
     }
-    const int nch = (x.m + c - 1) / c;
-    const int last = x.m - (nch - 1) * c;
-    const int mv = (nch - 1) * x.n + std::min(x.n, last);
-    if (!resident(qr_plan(mv, x.n, tcb))) {
-      rest.push_back(i);
-      continue;
-    }
+    const int nch = (x.m + c - 1) / c, mv = stacked(c);
     for (int j = 0; j < nch; ++j) {
       QrcpDesc q{};
       q.A = x.A + (long)j * c;
