@@ -15,6 +15,7 @@
 #include "common.h"
 #include "mlp.h"
 #include "pairs.cuh"
+#include "per_device.h"
 
 namespace ifmm {
 
@@ -310,8 +311,8 @@ struct MlpBuffers {
 static int mlp_ctas(int ns) { return std::min(152, (ns + kT - 1) / kT); }
 
 static void mlp_attrs() {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<std::once_flag> once;
+  std::call_once(once(), [] {
     CKM(cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mlp_smem_bytes(false)));
     CKM(cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mlp_smem_bytes(true)));
   });

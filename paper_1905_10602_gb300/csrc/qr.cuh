@@ -28,6 +28,7 @@
 
 #include "devmath.cuh"
 #include "fp64_ops.cuh"
+#include "per_device.h"
 #include "qr.h"
 
 namespace ifmm {
@@ -511,11 +512,10 @@ __global__ void __launch_bounds__(WARP ? 128 : 512, 1) k_qr_reg(const QrcpDesc* 
 template <typename TC, int E, bool PIV>
 bool qr_launch_e(const QrcpDesc* d, int nd, int R, int warps, size_t smem, cudaStream_t s, bool probe) {
   auto f = k_qr_reg<TC, E, qr_class_cols(E, sizeof(TC)), PIV, false>;
-  static bool attr = false;  // the attribute is per function and idempotent
-  if (!attr) {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [&] {
     if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
-    attr = true;
-  }
+  });
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nd * R), 1, 1);
   cfg.blockDim = dim3((unsigned)(32 * warps), 1, 1);

@@ -1,6 +1,7 @@
 // Every device kernel of the library lives in this translation unit: the
 // batched dense primitives (dense.cuh) and the IFMM-specific kernels below,
 // plus their launchers.
+#include <array>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -13,6 +14,7 @@
 #include "krylov.cuh"
 #include "biginv.cuh"
 #include "ifmm_kernels.h"
+#include "per_device.h"
 #include "qr.h"
 #include "runtime.h"
 
@@ -264,12 +266,11 @@ static void launch_gemm_tc(DescStage& st, const std::vector<GemmDesc>& v, int pr
     tp[i + 1] = tp[i] + (int)((long)((v[i].m + kTcBM - 1) / kTcBM) * ((v[i].n + kTcBN - 1) / kTcBN));
   const GemmDesc* d = st.push(v);
   const int* p = st.push(tp);
-  static bool attr = false;  // set once per process (the attribute is per function)
-  if (!attr) {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_gemm_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_tc_smem_bytes(0)));
     CK(cudaFuncSetAttribute(k_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_tc_smem_bytes(1)));
-    attr = true;
-  }
+  });
   prof_batch_tag() = (long)v.size();
   cudaEvent_t pe = profiler().begin(KK_GEMM32, st.stream);
   if (prec == P16)
@@ -387,8 +388,8 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
     req(v[i].A, span(v[i].n, v[i].n, v[i].ld), "inv.A", i);
     req(v[i].info, sizeof(int), "inv.info", i);
   }
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     auto set = [](const void* f) {
       CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem));
       if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
@@ -397,8 +398,10 @@ void launch_inv(DescStage& st, const std::vector<InvDesc>& v) {
     set((const void*)k_inv<1>);
     set((const void*)k_inv<2>);
   });
-  static int cl_ok[2][5] = {};  // per rows-per-thread and R = 1, 2, 4, 8, 16: 0 unknown, 1 yes, -1 no
+  // per rows-per-thread and R = 1, 2, 4, 8, 16: 0 unknown, 1 yes, -1 no
+  static PerDevice<std::array<std::array<int, 5>, 2>> cl_ok_of;
   static std::mutex cl_mu;
+  auto& cl_ok = cl_ok_of();
   // IFMM_INV_FALLBACK_N=n (read once per process; tests) sends every block of
   // at least n rows to the batched multi-CTA kernels
   static const int fallback_n = [] {
@@ -629,12 +632,13 @@ static std::vector<size_t> launch_qr_reg(DescStage& st, const std::vector<QrcpDe
   std::vector<size_t> rest;
   // whether a cluster of R CTAs can be resident (probed once per class and size)
   static std::mutex mu;
-  static int ok_cache[2][2][kQrClasses][17] = {};  // 0 unknown, 1 yes, -1 no
+  static PerDevice<std::map<std::array<int, 3>, int>> ok_of;  // 1 yes, -1 no, absent: unknown
+  auto& ok_cache = ok_of();
   auto resident = [&](const QrPlan& p) {
     if (p.cls < 0) return false;
     if (p.cls >= kQrClasses || p.R <= 8) return true;  // portable sizes
     std::lock_guard<std::mutex> lock(mu);
-    int& ok = ok_cache[prec == P32][PIV][p.cls][p.R];
+    int& ok = ok_cache[{prec, p.cls, p.R}];
     if (!ok) {
       auto go = qr_launcher(PIV, prec);
       ok = go(p.cls, nullptr, 1, p.R, 16, qr_reg_bytes(kQrRows[p.cls], 1024, 16 * p.R, tcb), st.stream, true)
@@ -736,8 +740,8 @@ void launch_qr(DescStage& st, const std::vector<QrDesc>& v, int prec) {
 void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
   if (v.empty()) return;
   for (auto& x : v) IFMM_REQUIRE(x.n <= 1024, IFMM_EINVAL, "pivoted QR wider than 1024 columns");
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_qrcp<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     CK(cudaFuncSetAttribute(k_qrcp<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   });
@@ -777,8 +781,8 @@ void launch_qrcp(DescStage& st, const std::vector<QrcpDesc>& v, int prec) {
 template <typename TC, int G, int EM>
 static void svd_rt_run(const SvdRtDesc* d, unsigned g, int R, int threads, int slot, cudaStream_t s) {
   static constexpr int cap = 220 * 1024;
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_svd_rt<TC, G, EM, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     if constexpr (sizeof(TC) == 8)
       CK(cudaFuncSetAttribute(k_svd_rt<TC, G, EM, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
@@ -932,12 +936,11 @@ void launch_m2l_init(DescStage& st, const std::vector<M2lChunk>& chunks, const M
   const int kk = prec == P64 ? KK_GEMM64 : KK_GEMM32;
   prof_batch_tag() = (long)chunks.size();
   cudaEvent_t pe = profiler().begin(kk, st.stream);
-  static bool attr = false;  // once per process: both instantiations may need > 48 KB
-  if (!attr) {
+  static PerDevice<std::once_flag> attr_once;  // both instantiations may need > 48 KB
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_m2l_init<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 64 * 64 * 8));
     CK(cudaFuncSetAttribute(k_m2l_init<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 64 * 64 * 4));
-    attr = true;
-  }
+  });
   const size_t smem = (size_t)4 * t.rc * t.rc * (prec == P64 ? 8 : 4);
   if (prec == P64)
     k_m2l_init<double><<<(unsigned)chunks.size(), 256, smem, st.stream>>>(d, (int)chunks.size(), t);
@@ -950,8 +953,8 @@ void launch_m2l_init(DescStage& st, const std::vector<M2lChunk>& chunks, const M
 void launch_il_transform(DescStage& st, const std::vector<int>& list, const IlTables& t, int md, int prec) {
   if (list.empty()) return;
   IFMM_REQUIRE(md >= 1 && md <= 64, IFMM_EINVAL, "IL transform tile out of range");
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_il_transform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 64 * 64 * 8));
     CK(cudaFuncSetAttribute(k_il_transform<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * 64 * 64 * 4));
   });
@@ -2044,8 +2047,8 @@ void launch_gram_sum(DescStage& st, const std::vector<double*>& dst, const std::
 void launch_chol(DescStage& st, const std::vector<double*>& mats, int r, double delta) {
   if (mats.empty()) return;
   IFMM_REQUIRE(r <= 128, IFMM_EINVAL, "Cholesky block too large");
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
+  static PerDevice<std::once_flag> attr_once;
+  std::call_once(attr_once(), [] {
     CK(cudaFuncSetAttribute(k_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, 140 * 1024));
   });
   double* const* d = st.push(mats);
@@ -2185,9 +2188,14 @@ void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, doub
   // CTAs of the panel's cluster: rows of at most two per thread and what shared
   // memory holds; 16 (a non-portable size) when the GPU can host it and the
   // matrix has rows enough for them
-  static std::once_flag once;
-  static int rmax = 0;
-  std::call_once(once, [] {
+  struct Panel {
+    std::once_flag once;
+    int rmax = 0;
+  };
+  static PerDevice<Panel> panel_of;
+  Panel& panel = panel_of();
+  int& rmax = panel.rmax;
+  std::call_once(panel.once, [&] {
     CK(cudaFuncSetAttribute(k_bi_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     CK(cudaFuncSetAttribute(k_bi_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kBiGemmBytes));
     rmax = 8;

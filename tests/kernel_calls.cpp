@@ -51,4 +51,54 @@ int kc_inv(int nmat, const int* n, double* A, int* info) {
     CK(cudaStreamDestroy(s));
   });
 }
+
+// one-sided Jacobi of the n x n matrix A (column-major), explicit (no pivoted R): the
+// sorted singular values and the normalised columns
+int kc_svd(int fp32, int n, const double* A, double* V, double* sig) {
+  return guarded([&] {
+    DescStage st;
+    cudaStream_t s;
+    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    st.stream = s;
+    DeviceArena mem;
+    const size_t nn = (size_t)n * n;
+    double *dA = mem.alloc(nn), *dV = mem.alloc(nn), *dw = mem.alloc(nn), *ds = mem.alloc(n);
+    int* dk = (int*)mem.alloc_bytes(sizeof(int));
+    CK(cudaMemcpyAsync(dA, A, sizeof(double) * nn, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(dk, &n, sizeof(int), cudaMemcpyHostToDevice, s));
+    SvdRtDesc d{};
+    d.A = dA;
+    d.ld = n;
+    d.n = n;
+    d.kin = dk;
+    d.jpvt = nullptr;
+    d.V = dV;
+    d.ldv = n;
+    d.sig = ds;
+    d.work = dw;
+    launch_svd_rt(st, std::vector<SvdRtDesc>{d}, fp32 ? P32 : P64);
+    CK(cudaMemcpyAsync(V, dV, sizeof(double) * nn, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(sig, ds, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    CK(cudaStreamDestroy(s));
+  });
+}
+
+// X = the inverse of the n x n matrix A (column-major) as the level-1 system's is formed
+int kc_top_inverse(int n, const double* A, double* X, int* info) {
+  return guarded([&] {
+    cudaStream_t s;
+    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    DeviceArena mem;
+    const size_t nn = (size_t)n * n;
+    double *dA = mem.alloc(nn), *dX = mem.alloc(nn), *dw = mem.alloc(big_inverse_work_doubles(n));
+    int *dp = (int*)mem.alloc_bytes(sizeof(int) * n), *di = (int*)mem.alloc_bytes(sizeof(int));
+    CK(cudaMemcpyAsync(dA, A, sizeof(double) * nn, cudaMemcpyHostToDevice, s));
+    big_inverse(s, dA, n, dX, dp, dw, di);
+    CK(cudaMemcpyAsync(X, dX, sizeof(double) * nn, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(info, di, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    CK(cudaStreamDestroy(s));
+  });
+}
 }
