@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "common.h"
 #include "mlp.h"
@@ -41,7 +42,9 @@ static void layer_offsets(int l, int* w, int* b) {
 // across all tiles of the CTA (exact products, two-sums: 10 FP32 operations
 // instead of one FP64 multiply-add, which occupies GB300's narrow FP64 pipe for
 // 64 FP32 slots), and are written once per CTA; k_mlp_reduce adds the CTAs'
-// parts in FP64 in CTA order.  Bound by the FP32 issue rate of those pair sums.
+// parts in FP64 in CTA order.  A CTA whose factors are too large or too small for
+// exact products in FP32's range (mlp_fits) does its tiles again with FP64 sums.
+// Bound by the FP32 issue rate of the pair sums.
 // 65,536 rows, one forward and one gradient call with their host copies: 0.83 ms,
 // against 75 ms for a kernel per layer whose weight gradient was one thread per
 // weight walking every row in FP64 (36 CTAs).
@@ -53,14 +56,55 @@ constexpr int kSmW2 = 0, kSmW3 = kSmW2 + 64 * kP, kSmW1 = kSmW3 + 64 * kP, kSmB 
               kSmDy = kSmX + kT * 9, kSmA = kSmDy + kT, kSmG = kSmA + 3 * kT * kP, kSmEnd = kSmG + 2 * kT * kP;
 constexpr int mlp_smem_bytes(bool grad) { return 4 * (grad ? kSmEnd : kSmG); }
 
-__device__ __forceinline__ void pair_mac(df& acc, float a, float b) {
+__device__ __forceinline__ void mac(df& acc, float a, float b) {
   const float p = a * b;
   const df s = df_two_sum(acc.h, p);
   acc.h = s.h;
   acc.l += s.l + fmaf(a, b, -p);
 }
-// C[s][j] = relu(b[j] + sum_i A[s][i] W[i][j]), i ascending
-__device__ __forceinline__ void mlp_hidden(const float* A, const float* W, const float* b, float* C, int tx, int ty) {
+__device__ __forceinline__ void mac(double& acc, float a, float b) { acc = fma((double)a, (double)b, acc); }
+__device__ __forceinline__ double sum_of(df v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double sum_of(double v) { return v; }
+
+// Smallest nonzero (less one, so that zeros do not count) and largest magnitude of a
+// set of floats, as bits.
+struct MlpRange {
+  unsigned lo = 0xffffffffu, hi = 0u;
+  __device__ __forceinline__ void add(float v) {
+    const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+    lo = min(lo, u - 1u);
+    hi = max(hi, u);
+  }
+};
+// Whether the factors a in A (and 1) and g in G of the CTA's threads can be multiplied
+// and summed as float pairs like FP64 would: finite, the last bit of every product a
+// multiple of 2^-149 (exponents from -103 on), and sums of 2^20 products below 2^127
+// (a CTA has at most 2^26 / 152 + 64 samples).  Every thread gets the answer.
+__device__ __forceinline__ bool mlp_fits(MlpRange A, MlpRange G) {
+  __shared__ unsigned r[4];
+  constexpr unsigned kAll = 0xffffffffu;
+  if (threadIdx.x < 4) r[threadIdx.x] = threadIdx.x & 1 ? 0u : kAll;
+  __syncthreads();
+  const unsigned v[4] = {__reduce_min_sync(kAll, A.lo), __reduce_max_sync(kAll, A.hi), __reduce_min_sync(kAll, G.lo),
+                         __reduce_max_sync(kAll, G.hi)};
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(r, v[0]);
+    atomicMax(r + 1, v[1]);
+    atomicMin(r + 2, v[2]);
+    atomicMax(r + 3, v[3]);
+  }
+  __syncthreads();
+  const unsigned ah = r[1], gh = r[3];
+  if (max(ah, gh) >= 0x7f800000u) return false;
+  if (gh == 0u) return true;
+  const int la = (int)((r[0] + 1u) >> 23) - 127, lg = (int)((r[2] + 1u) >> 23) - 127;
+  return (ah == 0u || la + lg >= -103) && max((int)(ah >> 23) - 127, 0) + (int)(gh >> 23) - 127 <= 105;
+}
+
+// C[s][j] = relu(b[j] + sum_i A[s][i] W[i][j]), i ascending; zero from sample cnt on
+// (a sample that is not there adds exact zeros to the gradient, whatever the weights)
+__device__ __forceinline__ void mlp_hidden(const float* A, const float* W, const float* b, float* C, int cnt, int tx,
+                                           int ty, MlpRange& rg) {
   float acc[4][2];
 #pragma unroll
   for (int u = 0; u < 4; ++u)
@@ -81,10 +125,15 @@ __device__ __forceinline__ void mlp_hidden(const float* A, const float* W, const
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) C[(ty + 16 * u) * kP + tx + 32 * v] = fmaxf(acc[u][v], 0.f);
+    for (int v = 0; v < 2; ++v) {
+      const float r = ty + 16 * u < cnt ? fmaxf(acc[u][v], 0.f) : 0.f;
+      C[(ty + 16 * u) * kP + tx + 32 * v] = r;
+      rg.add(r);
+    }
 }
 // D[s][i] = (sum_j G[s][j] W[i][j]) relu'(A[s][i]), j ascending
-__device__ __forceinline__ void mlp_back(const float* G, const float* W, const float* A, float* D, int tx, int ty) {
+__device__ __forceinline__ void mlp_back(const float* G, const float* W, const float* A, float* D, int tx, int ty,
+                                         MlpRange& rg) {
   float acc[4][2] = {};
 #pragma unroll 8
   for (int j = 0; j < 64; ++j) {
@@ -103,11 +152,14 @@ __device__ __forceinline__ void mlp_back(const float* G, const float* W, const f
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
       const int e = (ty + 16 * u) * kP + tx + 32 * v;
-      D[e] = A[e] > 0.f ? acc[u][v] : 0.f;
+      const float r = A[e] > 0.f ? acc[u][v] : 0.f;
+      D[e] = r;
+      rg.add(r);
     }
 }
 // acc[u][v] += sum_s A[s][ty + 16 u] G[s][tx + 32 v]
-__device__ __forceinline__ void mlp_outer(const float* A, const float* G, df (&acc)[4][2], int tx, int ty) {
+template <class ACC>
+__device__ __forceinline__ void mlp_outer(const float* A, const float* G, ACC (&acc)[4][2], int tx, int ty) {
 #pragma unroll 2
   for (int s = 0; s < kT; ++s) {
     float a[4], g[2];
@@ -118,39 +170,32 @@ __device__ __forceinline__ void mlp_outer(const float* A, const float* G, df (&a
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int v = 0; v < 2; ++v) pair_mac(acc[u][v], a[u], g[v]);
+      for (int v = 0; v < 2; ++v) mac(acc[u][v], a[u], g[v]);
   }
 }
 
-// y[s] (may be NULL with GRAD) for samples s < ns; GRAD: part[cta][IFMM_MLP_NWEIGHTS + 1] = the CTA's sums of the
-// gradient of L = mean (y - t)^2 / 2 and, last, of the samples' (y - t)^2 / 2
-template <bool GRAD>
-__global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w, const float* __restrict__ x,
-                                                     const float* __restrict__ t, float* __restrict__ y,
-                                                     double* __restrict__ part, int ns) {
-  extern __shared__ float sm[];
+// The CTA's tiles, weights staged (a barrier follows here): y[s] (may be NULL with GRAD)
+// for samples s < ns; GRAD: o[IFMM_MLP_NWEIGHTS + 1] = the CTA's sums of the gradient
+// of L = mean (y - t)^2 / 2, kept as ACC, and, last, of the samples' (y - t)^2 / 2.
+// Returns, in every thread, whether float pairs hold the sums (mlp_fits).
+template <bool GRAD, class ACC>
+__device__ __forceinline__ bool mlp_tiles(float* sm, const float* __restrict__ x, const float* __restrict__ t,
+                                          float* __restrict__ y, double* __restrict__ o, int ns) {
   float *W2 = sm + kSmW2, *W3 = sm + kSmW3, *W1 = sm + kSmW1, *B = sm + kSmB, *X = sm + kSmX, *dy = sm + kSmDy;
   float *A1 = sm + kSmA, *A2 = A1 + kT * kP, *A3 = A2 + kT * kP, *G2 = sm + kSmG, *G3 = G2 + kT * kP;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  for (int e = tid; e < 576; e += kMlpThreads) W1[e] = w[e];
-  for (int e = tid; e < 4096; e += kMlpThreads) {
-    W2[(e >> 6) * kP + (e & 63)] = w[640 + e];
-    W3[(e >> 6) * kP + (e & 63)] = w[4800 + e];
-  }
-  for (int e = tid; e < 64; e += kMlpThreads) {
-    B[e] = w[576 + e];
-    B[64 + e] = w[4736 + e];
-    B[128 + e] = w[8896 + e];
-    B[192 + e] = w[8960 + e];
-  }
-  if (tid == 0) B[256] = w[9024];
-  df w2[4][2] = {}, w3[4][2] = {}, w1[2] = {}, wb = {0.f, 0.f};
+  ACC w2[4][2] = {}, w3[4][2] = {}, w1[2] = {}, wb = {};
+  MlpRange ra, rg;
   double sq = 0.0;
   const int ntile = (ns + kT - 1) / kT;
   for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
     const int s0 = tile * kT, cnt = min(kT, ns - s0);
     __syncthreads();  // weights staged; the previous tile is done with X and dy
-    for (int e = tid; e < kT * 9; e += kMlpThreads) X[e] = e < cnt * 9 ? x[(long)s0 * 9 + e] : 0.f;
+    for (int e = tid; e < kT * 9; e += kMlpThreads) {
+      const float v = e < cnt * 9 ? x[(long)s0 * 9 + e] : 0.f;
+      X[e] = v;
+      ra.add(v);
+    }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -160,12 +205,14 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w
         float acc = B[j];
 #pragma unroll
         for (int i = 0; i < 9; ++i) acc = fmaf(X[s * 9 + i], W1[i * 64 + j], acc);
-        A1[s * kP + j] = fmaxf(acc, 0.f);
+        acc = s < cnt ? fmaxf(acc, 0.f) : 0.f;
+        A1[s * kP + j] = acc;
+        ra.add(acc);
       }
     __syncthreads();
-    mlp_hidden(A1, W2, B + 64, A2, tx, ty);
+    mlp_hidden(A1, W2, B + 64, A2, cnt, tx, ty, ra);
     __syncthreads();
-    mlp_hidden(A2, W3, B + 128, A3, tx, ty);
+    mlp_hidden(A2, W3, B + 128, A3, cnt, tx, ty, ra);
     __syncthreads();
     if (tid < kT) {
       float acc = B[256];
@@ -174,7 +221,9 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w
       if (y && tid < cnt) y[s0 + tid] = acc;
       if (GRAD) {
         const float d = tid < cnt ? acc - t[s0 + tid] : 0.f;
-        dy[tid] = d / (float)ns;
+        const float dn = d / (float)ns;
+        dy[tid] = dn;
+        rg.add(dn);
         sq += (double)(0.5f * d * d);
       }
     }
@@ -187,38 +236,39 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w
         for (int v = 0; v < 2; ++v) {
           const int e = (ty + 16 * u) * kP + tx + 32 * v;
           const float g = fmaf(dy[ty + 16 * u], B[192 + tx + 32 * v], 0.f);
-          G3[e] = A3[e] > 0.f ? g : 0.f;
+          const float r = A3[e] > 0.f ? g : 0.f;
+          G3[e] = r;
+          rg.add(r);
         }
       __syncthreads();
-      mlp_back(G3, W3, A2, G2, tx, ty);
+      mlp_back(G3, W3, A2, G2, tx, ty, rg);
       mlp_outer(A2, G3, w3, tx, ty);
       if (tid < 64) {
-        for (int s = 0; s < kT; ++s) pair_mac(wb, A3[s * kP + tid], dy[s]);
+        for (int s = 0; s < kT; ++s) mac(wb, A3[s * kP + tid], dy[s]);
       } else if (tid < 128) {
-        for (int s = 0; s < kT; ++s) pair_mac(wb, G3[s * kP + tid - 64], 1.f);
+        for (int s = 0; s < kT; ++s) mac(wb, G3[s * kP + tid - 64], 1.f);
       } else if (tid == 128) {
-        for (int s = 0; s < kT; ++s) pair_mac(wb, dy[s], 1.f);
+        for (int s = 0; s < kT; ++s) mac(wb, dy[s], 1.f);
       }
       __syncthreads();
       mlp_outer(A1, G2, w2, tx, ty);
       if (tid >= 160 && tid < 224)
-        for (int s = 0; s < kT; ++s) pair_mac(wb, G2[s * kP + tid - 160], 1.f);
+        for (int s = 0; s < kT; ++s) mac(wb, G2[s * kP + tid - 160], 1.f);
       __syncthreads();
-      mlp_back(G2, W2, A1, G3, tx, ty);  // G3 now holds the gradient of the first hidden layer
+      mlp_back(G2, W2, A1, G3, tx, ty, rg);  // G3 now holds the gradient of the first hidden layer
       __syncthreads();
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int e = tid + q * kMlpThreads;
         if (e < 576)
-          for (int s = 0; s < kT; ++s) pair_mac(w1[q], X[s * 9 + (e >> 6)], G3[s * kP + (e & 63)]);
+          for (int s = 0; s < kT; ++s) mac(w1[q], X[s * 9 + (e >> 6)], G3[s * kP + (e & 63)]);
       }
       if (tid >= 256 && tid < 320)
-        for (int s = 0; s < kT; ++s) pair_mac(wb, G3[s * kP + tid - 256], 1.f);
+        for (int s = 0; s < kT; ++s) mac(wb, G3[s * kP + tid - 256], 1.f);
     }
   }
   if constexpr (GRAD) {
-    double* o = part + (long)blockIdx.x * (IFMM_MLP_NWEIGHTS + 1);
-    auto put = [&](int e, df v) { o[e] = (double)v.h + (double)v.l; };
+    auto put = [&](int e, ACC v) { o[e] = sum_of(v); };
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -243,6 +293,38 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w
       for (int i = 0; i < kT; ++i) a += sqs[i];
       o[IFMM_MLP_NWEIGHTS] = a;
     }
+  }
+  if constexpr (GRAD && std::is_same<ACC, df>::value)
+    return mlp_fits(ra, rg);
+  else
+    return true;
+}
+
+template <bool GRAD>
+__global__ void __launch_bounds__(kMlpThreads) k_mlp(const float* __restrict__ w, const float* __restrict__ x,
+                                                     const float* __restrict__ t, float* __restrict__ y,
+                                                     double* __restrict__ part, int ns) {
+  extern __shared__ float sm[];
+  float *W2 = sm + kSmW2, *W3 = sm + kSmW3, *W1 = sm + kSmW1, *B = sm + kSmB;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < 576; e += kMlpThreads) W1[e] = w[e];
+  for (int e = tid; e < 4096; e += kMlpThreads) {
+    W2[(e >> 6) * kP + (e & 63)] = w[640 + e];
+    W3[(e >> 6) * kP + (e & 63)] = w[4800 + e];
+  }
+  for (int e = tid; e < 64; e += kMlpThreads) {
+    B[e] = w[576 + e];
+    B[64 + e] = w[4736 + e];
+    B[128 + e] = w[8896 + e];
+    B[192 + e] = w[8960 + e];
+  }
+  if (tid == 0) B[256] = w[9024];
+  if constexpr (GRAD) {
+    double* o = part + (long)blockIdx.x * (IFMM_MLP_NWEIGHTS + 1);
+    // where a factor is too large or too small for pairs, all over again in FP64
+    if (!mlp_tiles<true, df>(sm, x, t, y, o, ns)) mlp_tiles<true, double>(sm, x, t, y, o, ns);
+  } else {
+    mlp_tiles<false, df>(sm, x, t, y, nullptr, ns);
   }
 }
 static_assert(kSmA % 2 == 0, "the squares are stored as doubles");
