@@ -1247,28 +1247,42 @@ __device__ __forceinline__ float sqrt_fast(float x) {
 __device__ __forceinline__ bool svd_needs(float al, float be, float g) {
   return !(al < 1e-36f || be < 1e-36f || fabsf(g) <= 4e-7f * sqrt_fast(al) * sqrt_fast(be));
 }
+static __device__ __noinline__ bool svd_needs_rare(double al, double be, double g) {
+  return !(al < 1e-300 || be < 1e-300 || fabs(g) <= 1e-15 * sqrt(al) * sqrt(be));
+}
 __device__ __forceinline__ bool svd_needs(double al, double be, double g) {
-  return !(al < 1e-280 || be < 1e-280 || g * g <= 1e-30 * (al * be));
+  // below 2^-431 the products of the squares would underflow
+  if (min(dexp(al), dexp(be)) < 592) return svd_needs_rare(al, be, g);
+  return !(g * g <= 1e-30 * (al * be));
 }
 // rotation that orthogonalises columns of squared norms al, be and product g:
-// t = tan, c = cos, s = sin; t^2 + 2 z t - 1 = 0 with z = (be - al) / (2 g)
+// t = tan, c = cos, s = sin; t^2 + 2 z t - 1 = 0 with z = (be - al) / (2 g).  Columns
+// of very different size have a z whose square leaves the FP32 range: there 1 / (2 z)
+// is the tangent to far below rounding (relative error 1 / (4 z^2)).
 __device__ __forceinline__ void svd_rotation(float al, float be, float g, float& t, float& c, float& s) {
   const float z = __fdividef(be - al, g + g);
-  t = __fdividef(copysignf(1.f, z), fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
+  const bool far = fabsf(z) > 1e9f;
+  t = __fdividef(far ? 0.5f : copysignf(1.f, z), far ? z : fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
   const float x = fmaf(t, t, 1.f), y = rsqrtf(x);
   c = fmaf(0.5f * y, fmaf(-(x * y), y, 1.f), y);
   s = c * t;
 }
+static __device__ __noinline__ double quotient_rare(double a, double b) { return a / b; }
 __device__ __forceinline__ void svd_rotation(double al, double be, double g, double& t, double& c, double& s) {
   const double d = be - al, g2 = g + g;
-  const int sh = 1023 - max(dexp(d), dexp(g2));  // both into the FP32 range, exactly scaled
-  const float df = d2f_pow2(d, sh), gf = d2f_pow2(g2, sh);
-  const float z = __fdividef(df, gf);
-  const float t0 = __fdividef(copysignf(1.f, z), fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
-  t = f2d_pow2(t0, 0);
-  // one Newton step of g2 t^2 + 2 d t - g2 = 0: the residual in FP64
-  const double f = fma(t, fma(g2, t, d + d), -g2);
-  t -= f2d_pow2(__fdividef(d2f_pow2(f, sh), 2.f * fmaf(gf, t0, df)), 0);
+  const int ed = dexp(d), eg = dexp(g2);
+  if (ed - eg > 100) {  // g2 could leave the FP32 range below d
+    t = quotient_rare(g, d);
+  } else {
+    const int sh = 1023 - max(ed, eg);  // both into the FP32 range, exactly scaled
+    const float df = d2f_pow2(d, sh), gf = d2f_pow2(g2, sh);
+    const float z = __fdividef(df, gf);
+    const float t0 = __fdividef(copysignf(1.f, z), fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
+    t = f2d_pow2(t0, 0);
+    // one Newton step of g2 t^2 + 2 d t - g2 = 0: the residual in FP64
+    const double f = fma(t, fma(g2, t, d + d), -g2);
+    t -= f2d_pow2(__fdividef(d2f_pow2(f, sh), 2.f * fmaf(gf, t0, df)), 0);
+  }
   c = rsqrt_fp64(fma(t, t, 1.0));
   s = c * t;
 }
