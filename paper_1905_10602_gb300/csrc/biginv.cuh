@@ -1,6 +1,6 @@
 // The explicit inverse of one large FP64 matrix (the level-1 system): blocked
 // in-place Gauss-Jordan with partial pivoting, its rank-32 updates on the tensor
-// cores without loss of precision.
+// cores as products of 8-bit digits.
 //
 // A panel of nb = 32 columns K is exchanged on its own, rows spread over the CTAs
 // of one cluster; with P its pivot rows, B = A(P, K) and A' the exchanged panel
@@ -9,17 +9,26 @@
 // one product per panel.  Rows are never moved: after the last panel row p_k holds
 // x_k, so Ainv(k, p_k') = M(p_k, k') is written out at the end.
 //
-// The product is FP64-exact arithmetic on bfloat16 MMAs (the error-free splitting
-// of Ozaki, Ogita, Oishi and Rump): each row of A' and each column of A(P, J) is
-// scaled by a power of two to |m| < 1 and cut into seven signed 8-bit digits (55
-// bits of the largest entry); products of digits summed over 32 terms and up to
-// seven digit pairs stay below 2^22, so the FP32 accumulators are exact integers,
-// and the eight orders i + j <= 7 are added up in 64-bit integers (what is dropped
-// is below 2^-58 of the largest term).  34 MMA passes replace the FP64
-// multiply-adds, whose pipe (2 per clock and SM) bounds the plain elimination: n =
-// 3,628 needs 90 ms there.  What bounds it now is the panels' chain of n pivot
-// steps (one cluster barrier each).  The two launches per column it replaces: n =
-// 3,628 243 -> 52 ms, n = 2,296 69 -> 18, n = 1,417 29 -> 7.9.
+// The product splits its operands into digits (the error-free splitting of Ozaki,
+// Ogita, Oishi and Rump): each row of A' and each column of A(P, J) is scaled by a
+// power of two to |m| < 1 and rounded to seven signed 8-bit digits, 55 bits below
+// that power; products of digits summed over 32 terms and up to seven digit pairs
+// stay below 2^22, so the FP32 accumulators are exact integers, and the eight
+// orders i + j <= 7 are added up in 64-bit integers.  With r and c the largest
+// entries of a row of A' and a column of A(P, J), the operands' rounding leaves
+// 32 * 2^-54 r c over the 32 terms at most and the dropped orders 2^-54.7 r c: the
+// error is relative to r c, not to the terms, and an entry 2^-k below its row's or
+// column's largest keeps 55 - k bits.  Rows of very different size would put the
+// large entries of A' against the small ones of A(P, J) (A' is graded by 1/d_p, A(P, J)
+// by d_p), so column p of A' is taken times 2^s_p and row p of A(P, J) times 2^-s_p, s_p
+// the exponent of the largest entry of row p of the matrix: what a power-of-two
+// scaling of the rows would give, with the pivots of the unscaled matrix.  (The
+// columns' sizes cancel without it.)  Half the rows times 2^-40, n = 200, emulated in
+// NumPy: error 3.8e10 u |X||A||X| without, 0.4 u with, 0.5 u in plain FP64 elimination.
+// 34 MMA passes replace the FP64 multiply-adds, whose pipe (2 per clock and SM)
+// bounds the plain elimination: n = 3,628 needs 90 ms there.  What bounds it now is
+// the panels' chain of n pivot steps (one cluster barrier each).  The two launches
+// per column it replaces: n = 3,628 243 -> 52 ms, n = 2,296 69 -> 18, n = 1,417 29 -> 7.9.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -43,17 +52,37 @@ inline int bi_rows(int n, int R) { return (n + R - 1) / R; }
 inline size_t bi_panel_bytes(int n, int R) {
   return (size_t)bi_rows(n, R) * (kBiNb + 1) * sizeof(double) + (size_t)2 * R * (kBiNb + 2) * sizeof(double);
 }
-// device scratch: digits of A' and of the pivot rows (n x 32 each and slice), their exponents, the used rows
+// device scratch: digits of A' and of the pivot rows (n x 32 each and slice), their exponents, the rows' scales, the
+// used rows
 inline size_t bi_work_bytes(int n) {
   const size_t np = ((size_t)n + kBiTile - 1) / kBiTile * kBiTile;
-  return 2 * kBiSlices * np * kBiNb * 2 + 2 * np * sizeof(int) + np + 1024;
+  return 2 * kBiSlices * np * kBiNb * 2 + 3 * np * sizeof(int) + np + 1024;
 }
 struct BiWork {
   uint16_t *da, *db;  // digits [slice][row or column][32], bfloat16
   int *ea, *eb;       // exponents
+  int* es;            // biased exponent of the largest entry of each row of the matrix
   unsigned char* used;
   int np;             // rows and columns, padded to the tile
 };
+
+constexpr int kBiNone = -0x100000;  // no nonzero entry
+
+// The power of two that row p counts as (its largest entry's; an infinity or NaN, or
+// nothing but zeros and subnormals: 1)
+__device__ __forceinline__ int bi_scale(const BiWork& w, int p) {
+  const int e = w.es[p];
+  return e > 0 && e < 2047 ? e - 1023 : 0;
+}
+// es (zeroed) = the rows' largest biased exponents; a thread per row, 64 columns a CTA
+__global__ void __launch_bounds__(256) k_bi_scales(const double* __restrict__ A, int n, BiWork w) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const int j1 = min(n, (int)(blockIdx.y + 1) * 64);
+  int e = 0;
+  for (int j = blockIdx.y * 64; j < j1; ++j) e = max(e, dexp(A[i + (long)j * n]));
+  atomicMax(w.es + i, e);
+}
 
 // The seven digits of x / 2^e (|x| < 2^e) as bfloat16 bits: d[s] has weight
 // 2^(-7 - 8 s); rounded to 55 bits.
@@ -92,6 +121,7 @@ __global__ void __launch_bounds__(kBiThreads) k_bi_panel(double* __restrict__ A,
   int* ki = (int*)(kv + 2 * R);               // [2][R] rows
   __shared__ unsigned rh[16], rl[16];
   __shared__ int ri[16];
+  __shared__ int sx[kBiNb];  // the panel's pivot rows, then their scales
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   for (int c = wp; c < kBiNb; c += kBiThreads / 32)
     for (int i = lane; i < ml; i += 32) P[(size_t)c * chunk + i] = c < kb ? A[(r0 + i) + (long)(k0 + c) * n] : 0.0;
@@ -155,7 +185,10 @@ __global__ void __launch_bounds__(kBiThreads) k_bi_panel(double* __restrict__ A,
       bad = k0 + k + 1;
       break;
     }
-    if (rank == 0 && tid == 0) piv[k0 + k] = p;
+    if (tid == 0) {
+      sx[k] = p;
+      if (rank == 0) piv[k0 + k] = p;
+    }
     const double* row = rowb + (b * R + p / chunk) * kBiNb;
     const int pl = p - r0;  // the pivot's local row, if it is here
 #pragma unroll
@@ -181,6 +214,8 @@ __global__ void __launch_bounds__(kBiThreads) k_bi_panel(double* __restrict__ A,
     cl.sync();
     return;
   }
+  if (tid < kBiNb) sx[tid] = tid < kb ? bi_scale(w, sx[tid]) : 0;
+  __syncthreads();
   for (int c = wp; c < kb; c += kBiThreads / 32)
     for (int i = lane; i < ml; i += 32) A[(r0 + i) + (long)(k0 + c) * n] = P[(size_t)c * chunk + i];
 #pragma unroll
@@ -188,16 +223,22 @@ __global__ void __launch_bounds__(kBiThreads) k_bi_panel(double* __restrict__ A,
     const int i = tid + v * kBiThreads;
     if (i >= ml) continue;
     w.used[r0 + i] = used[v];
-    // digits of row r0 + i
-    int e = 0;
-    for (int c = 0; c < kBiNb; ++c) e = max(e, dexp(P[(size_t)c * chunk + i]));
-    w.ea[r0 + i] = e == 2047 ? kBiBad : e - 1022;
+    // digits of row r0 + i, entry c times 2^sx[c]
+    int e = kBiNone;
+    bool fin = true;
+    for (int c = 0; c < kBiNb; ++c) {
+      const int ex = dexp(P[(size_t)c * chunk + i]);
+      fin = fin && ex < 2047;
+      if (ex > 0) e = max(e, ex + sx[c]);
+    }
+    if (e == kBiNone) e = 0;
+    w.ea[r0 + i] = fin ? e - 1022 : kBiBad;
     for (int c0 = 0; c0 < kBiNb; c0 += 8) {
       unsigned lo16[kBiSlices][4];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         unsigned d[kBiSlices];
-        bi_digits(e == 2047 ? 0.0 : P[(size_t)(c0 + u) * chunk + i], e - 1022, d);
+        bi_digits(fin ? P[(size_t)(c0 + u) * chunk + i] : 0.0, e - 1022 - sx[c0 + u], d);
 #pragma unroll
         for (int s = 0; s < kBiSlices; ++s) lo16[s][u >> 1] = (u & 1) ? lo16[s][u >> 1] | d[s] << 16 : d[s];
       }
@@ -211,7 +252,7 @@ __global__ void __launch_bounds__(kBiThreads) k_bi_panel(double* __restrict__ A,
 }
 
 // Digits of the pivot rows of panel k0 in every other column (a warp per column,
-// lane s: row piv[k0 + s]), which are then zero; the panel's own columns get zero
+// lane s: row p = piv[k0 + s], times 2^-s_p), which are then zero; the panel's own columns get zero
 // digits (their product must add nothing).
 __global__ void __launch_bounds__(256) k_bi_rows(double* __restrict__ A, int n, int k0, int kb,
                                                  const int* __restrict__ piv, BiWork w, const int* __restrict__ info) {
@@ -220,15 +261,21 @@ __global__ void __launch_bounds__(256) k_bi_rows(double* __restrict__ A, int n, 
   if (j >= w.np) return;
   const bool own = j >= n || (j >= k0 && j < k0 + kb);
   double x = 0.0;
+  int sc = 0;
   if (!own && lane < kb) {
-    double* a = A + piv[k0 + lane] + (long)j * n;
+    const int p = piv[k0 + lane];
+    double* a = A + p + (long)j * n;
+    sc = bi_scale(w, p);
     x = *a;
     *a = 0.0;
   }
-  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)dexp(x));
-  if (lane == 0) w.eb[j] = e == 2047 ? kBiBad : e - 1022;
+  const int ex = dexp(x);
+  const bool fin = __all_sync(0xffffffffu, ex < 2047);
+  int e = __reduce_max_sync(0xffffffffu, ex > 0 ? ex - sc : kBiNone);
+  if (e == kBiNone) e = 0;
+  if (lane == 0) w.eb[j] = fin ? e - 1022 : kBiBad;
   unsigned d[kBiSlices];
-  bi_digits(e == 2047 ? 0.0 : x, e - 1022, d);
+  bi_digits(fin ? x : 0.0, e - 1022 + sc, d);
 #pragma unroll
   for (int s = 0; s < kBiSlices; ++s) w.db[((size_t)s * w.np + j) * kBiNb + lane] = (uint16_t)d[s];
 }

@@ -56,9 +56,12 @@ void launch_chol(DescStage& st, const std::vector<double*>& mats, int r, double 
 void launch_gather_perm(cudaStream_t s, const double* src, const int* perm, double* dst, int n, int dof = 1);
 void launch_scatter_perm(cudaStream_t s, const double* src, const int* perm, double* dst, int n, int dof = 1);
 // out (ld n) = the inverse of the n x n matrix M (overwritten); piv: n ints, work:
-// big_inverse_work_doubles(n), info: 0, or k + 1 when step k found no nonzero pivot
+// big_inverse_work_doubles(n), info: 0, or k + 1 when step k found no nonzero pivot;
+// columns: by two launches per column whatever n is (what a matrix takes whose panels
+// fit no cluster, n above 13,120)
 size_t big_inverse_work_doubles(int n);
-void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, double* d_work, int* d_info);
+void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, double* d_work, int* d_info,
+                 bool columns = false);
 // phase-B basis changes of the touched IL entries `list` (every rank <= md <= 64)
 void launch_il_transform(DescStage& st, const std::vector<int>& list, const IlTables& t, int md, int prec);
 // level-start M2L blocks T'_a K T_b of the entries grouped by offset (rc <= 64)

@@ -2183,7 +2183,8 @@ static void big_inverse_columns(cudaStream_t s, double* A, int ld, int n, int* d
 
 size_t big_inverse_work_doubles(int n) { return std::max((bi_work_bytes(n) + 7) / 8, (size_t)2 * n); }
 
-void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, double* d_work, int* d_info) {
+void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, double* d_work, int* d_info,
+                 bool columns) {
   CK(cudaMemsetAsync(d_info, 0, sizeof(int), s));
   // CTAs of the panel's cluster: rows of at most two per thread and what shared
   // memory holds; 16 (a non-portable size) when the GPU can host it and the
@@ -2220,7 +2221,7 @@ void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, doub
   int R = 1;
   while (R < rmax && bi_rows(n, R) > 32) R *= 2;
   cudaEvent_t pe = profiler().begin(KK_GJ_BIG, s, 1);
-  if (bi_rows(n, R) > 2 * kBiThreads || bi_panel_bytes(n, R) > (size_t)220 * 1024) {
+  if (columns || bi_rows(n, R) > 2 * kBiThreads || bi_panel_bytes(n, R) > (size_t)220 * 1024) {
     big_inverse_columns(s, M, n, n, d_piv, d_work, d_info);
     CK(cudaMemcpyAsync(out, M, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
     profiler().end(KK_GJ_BIG, s, pe);
@@ -2232,8 +2233,10 @@ void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, doub
   w.db = w.da + (size_t)kBiSlices * w.np * kBiNb;
   w.ea = (int*)(w.db + (size_t)kBiSlices * w.np * kBiNb);
   w.eb = w.ea + w.np;
-  w.used = (unsigned char*)(w.eb + w.np);
-  CK(cudaMemsetAsync(w.used, 0, w.np, s));
+  w.es = w.eb + w.np;
+  w.used = (unsigned char*)(w.es + w.np);
+  CK(cudaMemsetAsync(w.es, 0, w.np * (sizeof(int) + 1), s));  // es and used
+  k_bi_scales<<<dim3((unsigned)((n + 255) / 256), (unsigned)((n + 63) / 64)), 256, 0, s>>>(M, n, w);
   CK(cudaMemsetAsync(w.da, 0, sizeof(uint16_t) * (size_t)kBiSlices * w.np * kBiNb, s));  // the padding rows
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)R);
@@ -2247,7 +2250,7 @@ void big_inverse(cudaStream_t s, double* M, int n, double* out, int* d_piv, doub
   cfg.attrs = at;
   cfg.numAttrs = 1;
   const unsigned tiles = (unsigned)(w.np / kBiTile);
-  long launches = 0;
+  long launches = 1;
   for (int k0 = 0; k0 < n; k0 += kBiNb) {
     const int kb = std::min(kBiNb, n - k0);
     CK(cudaLaunchKernelEx(&cfg, k_bi_panel, M, n, k0, kb, d_piv, w, d_info));

@@ -84,8 +84,9 @@ int kc_svd(int fp32, int n, const double* A, double* V, double* sig) {
   });
 }
 
-// X = the inverse of the n x n matrix A (column-major) as the level-1 system's is formed
-int kc_top_inverse(int n, const double* A, double* X, int* info) {
+// X = the inverse of the n x n matrix A (column-major) as the level-1 system's is
+// formed; columns: by the launches per column
+int kc_top_inverse(int n, const double* A, double* X, int* info, int columns) {
   return guarded([&] {
     cudaStream_t s;
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
@@ -94,7 +95,7 @@ int kc_top_inverse(int n, const double* A, double* X, int* info) {
     double *dA = mem.alloc(nn), *dX = mem.alloc(nn), *dw = mem.alloc(big_inverse_work_doubles(n));
     int *dp = (int*)mem.alloc_bytes(sizeof(int) * n), *di = (int*)mem.alloc_bytes(sizeof(int));
     CK(cudaMemcpyAsync(dA, A, sizeof(double) * nn, cudaMemcpyHostToDevice, s));
-    big_inverse(s, dA, n, dX, dp, dw, di);
+    big_inverse(s, dA, n, dX, dp, dw, di, columns != 0);
     CK(cudaMemcpyAsync(X, dX, sizeof(double) * nn, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(info, di, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

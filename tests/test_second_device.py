@@ -26,7 +26,7 @@ def svd(prec, n):
 
 def top(n):
     A, X, info = np.zeros((n, n)), np.zeros((n, n)), np.zeros(1, np.int32)
-    assert kc.kc_top_inverse(n, vp(A), vp(X), vp(info)) == 0
+    assert kc.kc_top_inverse(n, vp(A), vp(X), vp(info), 0) == 0
 
 calls = [
     lambda: ifmm.ifmm_mlp_forward(w, x),
