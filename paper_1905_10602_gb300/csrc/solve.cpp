@@ -329,10 +329,21 @@ static std::mutex g_tune_mutex;
 // The float-pair matvec's tile for a tree: the autotuner's choice, remembered
 // per device and point count for the life of the process, so that trees of a
 // size already seen (a new tree per problem, as in a time loop) skip the
-// timing runs (fifteen launches of the full product).
+// timing runs (three launches of the full product per candidate).  short_of_memory:
+// the symmetric kernel's buffer did not fit this time (part is null); the choice
+// among the full sums is remembered on its own, so that the next call with room
+// takes the symmetric kernel again.
 static int matvec_tile(ifmm_tree* tm, cudaStream_t s, const float* q, const double* in, double* out, int64_t N,
-                       const ifmm_kernel* k, float2* part) {
+                       const ifmm_kernel* k, float2* part, bool short_of_memory) {
   std::lock_guard<std::mutex> lock(g_tune_mutex);
+  static std::map<std::pair<int, int64_t>, int> seen, seen_full;
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (short_of_memory) {
+    int& code = seen_full[{dev, N}];
+    if (!code) code = autotune_matvec_df(s, tm->d_pts_df, q, q + N, in, out, (int)N, k->scale, k->diag, nullptr);
+    return code;
+  }
   if (tm->matvec_block) return tm->matvec_block;
   // IFMM_MATVEC_TILE (read when a tree first needs its tile) forces a kernel:
   // "sym" or "sym2" (tiles of 128 or 256 points), or "<threads>x<targets per thread>" (128x1, 256x1, 512x1, 128x2,
@@ -351,9 +362,6 @@ static int matvec_tile(ifmm_tree* tm, cudaStream_t s, const float* q, const doub
     tm->matvec_block_v = {code & 0xffff, code >> 16};
     return code;
   }
-  static std::map<std::pair<int, int64_t>, int> seen;
-  int dev = 0;
-  CK(cudaGetDevice(&dev));
   auto it = seen.find({dev, N});
   const int code = it != seen.end()
                        ? it->second
@@ -467,7 +475,7 @@ static double* get_or_null(Vecs& W, size_t n) {
 
 // doubles of the partial-sum buffer of the symmetric float-pair matvec, when it
 // is at most 8 GiB (N up to about 300,000 points) and this tree may take that
-// kernel; 0 otherwise
+// kernel; 0 otherwise (a product that finds no room for it takes the full sums)
 static size_t sym_part_doubles(const ifmm_tree& t) {
   if (t.matvec_block && (t.matvec_block >> 16) != 3) return 0;
   const size_t floats = matvec_sym_part_floats((int)t.N);
@@ -573,7 +581,6 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
     const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
     Vecs V, W;
     for (int i = 0; i < (df_mv ? 4 : 3); ++i) V.reserve(N);
-    if (df_mv && np) V.reserve(np);
     double* a = V.get(N);
     double* b = V.get(N);
     double* c = V.get(N);
@@ -590,8 +597,11 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
       float* q = (float*)V.get(N);
       launch_split_df(s, a, q, q + N, (int)N);
       ifmm_tree* tm = const_cast<ifmm_tree*>(t);
-      float2* part = np ? (float2*)V.get(np) : nullptr;
-      const int tile = tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, q, a, b, N, k, part);
+      float2* part = np ? (float2*)get_or_null(W, np) : nullptr;
+      const bool short_of_memory = np && !part;
+      const int tile = tm->matvec_block && !short_of_memory
+                           ? tm->matvec_block
+                           : matvec_tile(tm, s, q, a, b, N, k, part, short_of_memory);
       launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, part);
     } else {
       launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? get_or_null(W, np) : nullptr);
@@ -641,7 +651,6 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     Vm.reserve(2 * (size_t)m + 2);
     Vm.reserve(nkp);
     if (df_mv) Vm.reserve(N);
-    if (df_mv && np) Vm.reserve(np);
     double* bt = Vm.get(N);   // b in tree order
     double* xt = Vm.get(N);   // x in tree order
     double* rt = Vm.get(N);
@@ -652,7 +661,7 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     double* kp = Vm.get(nkp);
     double* tmp = Vm.get(N);
     float* qdf = df_mv ? (float*)Vm.get(N) : nullptr;
-    double* part = !np ? nullptr : (df_mv ? Vm.get(np) : get_or_null(W, np));
+    double* part = np ? get_or_null(W, np) : nullptr;
     const double* src = b;
     if (!dev) {
       CK(cudaMemcpyAsync(tmp, b, sizeof(double) * N, cudaMemcpyHostToDevice, s));
@@ -677,8 +686,10 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
       } else if (df_mv) {
         launch_split_df(s, in, qdf, qdf + N, (int)N);
         ifmm_tree* tm = const_cast<ifmm_tree*>(t);
-        const int tile =
-            tm->matvec_block ? tm->matvec_block : matvec_tile(tm, s, qdf, in, out, N, k, (float2*)part);
+        const bool short_of_memory = np && !part;
+        const int tile = tm->matvec_block && !short_of_memory
+                             ? tm->matvec_block
+                             : matvec_tile(tm, s, qdf, in, out, N, k, (float2*)part, short_of_memory);
         launch_matvec_df(s, t->d_pts_df, qdf, qdf + N, in, out, (int)N, k->scale, k->diag, tile, (float2*)part);
       } else {
         launch_matvec(s, t->d_pts, (int)NP, in, out, *k, part);
