@@ -25,6 +25,11 @@
  *     singular pivots, GMRES convergence, host outputs); otherwise they may
  *     return early.
  *   - A handle must not be used from two threads at the same time.
+ *   - Memory between calls: the library keeps device blocks of finished calls for
+ *     the next one, at most 16 GiB of them unused per device (and 256 MiB of pinned
+ *     host memory).  Other allocators of the process cannot claim them; they are
+ *     given back when an allocation of the library's own would fail without them, and
+ *     all of them when the last tree that was used on a device is freed.
  *   - There is no CPU fallback: without a CUDA device every compute call
  *     returns IFMM_ECUDA.
  */

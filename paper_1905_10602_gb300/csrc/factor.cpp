@@ -230,7 +230,7 @@ struct Factorizer {
     gprec = F.o.precision == IFMM_PREC_BF16 ? P16 : prec;
     if (F.o.rank_mode == IFMM_RANK_LEARNED) {
       IFMM_REQUIRE(F.o.mlp != nullptr, IFMM_EINVAL, "learned rank mode needs the MLP weights");
-      CK(cudaMalloc(&d_mlp, sizeof(float) * IFMM_MLP_NWEIGHTS));
+      CK(device_malloc((void**)&d_mlp, sizeof(float) * IFMM_MLP_NWEIGHTS));
       CK(cudaMemcpy(d_mlp, F.o.mlp, sizeof(float) * IFMM_MLP_NWEIGHTS, cudaMemcpyHostToDevice));
     }
     if (F.o.rank_mode == IFMM_RANK_REPLAY) {
@@ -1231,7 +1231,7 @@ struct Factorizer {
         registry().remove_range(d_info, sizeof(int) * info_cap);
         cudaFree(d_info);
       }
-      CK(cudaMalloc(&d_info, sizeof(int) * std::max(ng, 64)));
+      CK(device_malloc((void**)&d_info, sizeof(int) * std::max(ng, 64)));
       info_cap = std::max(ng, 64);
       registry().add(d_info, sizeof(int) * info_cap);
     }

@@ -17,6 +17,7 @@
 #include "mlp.h"
 #include "pairs.cuh"
 #include "per_device.h"
+#include "runtime.h"
 
 namespace ifmm {
 
@@ -375,7 +376,7 @@ struct MlpBuffers {
   char* base = nullptr;
   size_t off = 0;
   static size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
-  explicit MlpBuffers(size_t bytes) { CKM(cudaMalloc((void**)&base, std::max<size_t>(bytes, 256))); }
+  explicit MlpBuffers(size_t bytes) { CKM(device_malloc((void**)&base, std::max<size_t>(bytes, 256))); }
   MlpBuffers(const MlpBuffers&) = delete;
   MlpBuffers& operator=(const MlpBuffers&) = delete;
   ~MlpBuffers() { cudaFree(base); }

@@ -56,7 +56,28 @@ void drop_pinned(State& S) {
   S.pinned_bytes = 0;
 }
 
+// gives the device memory kept unused on dev back to the driver
+void trim(State& S, int dev) {
+  auto it = S.dev.find(dev);
+  if (it == S.dev.end() || !it->second.pool) return;
+  cudaStreamSynchronize(it->second.stream);
+  cudaMemPoolTrimTo(it->second.pool, 0);
+}
+
 }  // namespace
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  State& S = state();
+  std::lock_guard<std::mutex> lock(S.mu);
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) trim(S, dev);
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 
 void* pool_alloc(size_t bytes) {
   State& S = state();
@@ -68,8 +89,7 @@ void* pool_alloc(size_t bytes) {
   cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, P.pool, P.stream);
   if (e == cudaErrorMemoryAllocation) {  // give back what is kept and try once more
     cudaGetLastError();
-    cudaStreamSynchronize(P.stream);
-    cudaMemPoolTrimTo(P.pool, 0);
+    trim(S, dev);
     e = cudaMallocFromPoolAsync(&p, bytes, P.pool, P.stream);
   }
   if (e != cudaSuccess) cudaGetLastError();
@@ -111,7 +131,17 @@ void* pinned_alloc(size_t bytes, size_t* got) {
     }
   }
   void* p = nullptr;
-  CK(cudaMallocHost(&p, bytes));
+  cudaError_t e = cudaMallocHost(&p, bytes);
+  if (e == cudaErrorMemoryAllocation) {  // give back what is kept and try once more
+    cudaGetLastError();
+    {
+      std::lock_guard<std::mutex> lock(S.mu);
+      drop_pinned(S);
+    }
+    e = cudaMallocHost(&p, bytes);
+  }
+  if (e != cudaSuccess) cudaGetLastError();
+  CK(e);
   *got = bytes;
   return p;
 }
@@ -136,10 +166,7 @@ void pool_tree_count(int delta) {
   S.trees += delta;
   if (S.trees > 0) return;
   drop_pinned(S);
-  for (auto& d : S.dev) {
-    cudaStreamSynchronize(d.second.stream);
-    cudaMemPoolTrimTo(d.second.pool, 0);
-  }
+  for (auto& d : S.dev) trim(S, d.first);
 }
 
 void pool_quiesce() {

@@ -2530,9 +2530,9 @@ ifmm_status ifmm_convert_check(const double* x, int64_t n, int shift, float* f, 
     if (n == 0) return IFMM_OK;
     double *dx = nullptr, *db = nullptr;
     float* df = nullptr;
-    CK(cudaMalloc(&dx, sizeof(double) * n));
-    CK(cudaMalloc(&db, sizeof(double) * n));
-    CK(cudaMalloc(&df, sizeof(float) * n));
+    CK(ifmm::device_malloc((void**)&dx, sizeof(double) * n));
+    CK(ifmm::device_malloc((void**)&db, sizeof(double) * n));
+    CK(ifmm::device_malloc((void**)&df, sizeof(float) * n));
     cudaError_t e = cudaMemcpy(dx, x, sizeof(double) * n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
       ifmm::k_conv_check<<<(unsigned)((n + 255) / 256), 256>>>(dx, (int)n, shift, df, db);

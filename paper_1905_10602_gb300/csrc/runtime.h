@@ -68,7 +68,8 @@ void poison_fill(void* p, size_t bytes);
 // for a workspace, 0.3 ms for a 256 MB chunk, 3.2 ms for 64 MB of pinned memory;
 // a job takes a few dozen).  Bounded: at most 16 GiB of unused device memory (of 280) and
 // 256 MiB of unused pinned memory stay, and all of it is given back when the
-// process' last tree is freed, or when an allocation fails for want of memory.
+// process' last tree is freed, or when one of the library's own allocations fails for
+// want of memory.
 // Safe from any thread and stream: a block is handed out free of pending work,
 // and pool_free / pinned_free are only called once the work that used the block
 // has finished (see pool_quiesce).
@@ -77,6 +78,9 @@ void pool_free(void* p);
 void* pinned_alloc(size_t bytes, size_t* got);  // at least bytes; *got = the chunk's size
 void pinned_free(void* p, size_t got);
 void pool_tree_count(int delta);           // live trees of the process
+// cudaMalloc for what outlives the pool's purpose (a tree's copies, weights): what the
+// pool keeps unused on the current device is given back before it reports no memory
+cudaError_t device_malloc(void** p, size_t bytes);
 // For releases while an exception passes: work that was issued may still use
 // the memory, so the device is waited for first.
 void pool_quiesce();

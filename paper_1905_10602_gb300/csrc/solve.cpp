@@ -396,10 +396,10 @@ void ifmm_tree::ensure_device() {
   std::vector<double> soa(3 * (size_t)N);
   for (int64_t i = 0; i < N; ++i)
     for (int d = 0; d < 3; ++d) soa[(size_t)d * N + i] = pts[3 * i + d];
-  CK(cudaMalloc(&d_pts, sizeof(double) * 3 * N));
+  CK(device_malloc((void**)&d_pts, sizeof(double) * 3 * N));
   pool_tree_count(1);
   CK(cudaMemcpy(d_pts, soa.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&d_perm, sizeof(int32_t) * N));
+  CK(device_malloc((void**)&d_perm, sizeof(int32_t) * N));
   CK(cudaMemcpy(d_perm, perm.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
   std::vector<float> dfp(6 * (size_t)N);
   for (int64_t i = 0; i < N; ++i)
@@ -409,7 +409,7 @@ void ifmm_tree::ensure_device() {
       dfp[(size_t)(2 * d) * N + i] = h;
       dfp[(size_t)(2 * d + 1) * N + i] = (float)(v - (double)h);
     }
-  CK(cudaMalloc(&d_pts_df, sizeof(float) * 6 * N));
+  CK(device_malloc((void**)&d_pts_df, sizeof(float) * 6 * N));
   CK(cudaMemcpy(d_pts_df, dfp.data(), sizeof(float) * 6 * N, cudaMemcpyHostToDevice));
   registry().add(d_pts, sizeof(double) * 3 * N);
   registry().add(d_perm, sizeof(int32_t) * N);
