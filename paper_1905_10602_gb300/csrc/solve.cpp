@@ -385,6 +385,26 @@ static bool is_device_ptr(const void* p) {
 
 using namespace ifmm;
 
+// the tree's device copies, as far as they exist
+static void release_device(ifmm_tree& t) {
+  if (t.d_pts) {
+    registry().remove_range(t.d_pts, sizeof(double) * 3 * t.N);
+    cudaFree(t.d_pts);
+    t.d_pts = nullptr;
+    pool_tree_count(-1);
+  }
+  if (t.d_perm) {
+    registry().remove_range(t.d_perm, sizeof(int32_t) * t.N);
+    cudaFree(t.d_perm);
+    t.d_perm = nullptr;
+  }
+  if (t.d_pts_df) {
+    registry().remove_range(t.d_pts_df, sizeof(float) * 6 * t.N);
+    cudaFree(t.d_pts_df);
+    t.d_pts_df = nullptr;
+  }
+}
+
 void ifmm_tree::ensure_device() {
   if (d_pts) return;
   int ndev = 0;
@@ -396,11 +416,6 @@ void ifmm_tree::ensure_device() {
   std::vector<double> soa(3 * (size_t)N);
   for (int64_t i = 0; i < N; ++i)
     for (int d = 0; d < 3; ++d) soa[(size_t)d * N + i] = pts[3 * i + d];
-  CK(device_malloc((void**)&d_pts, sizeof(double) * 3 * N));
-  pool_tree_count(1);
-  CK(cudaMemcpy(d_pts, soa.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice));
-  CK(device_malloc((void**)&d_perm, sizeof(int32_t) * N));
-  CK(cudaMemcpy(d_perm, perm.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
   std::vector<float> dfp(6 * (size_t)N);
   for (int64_t i = 0; i < N; ++i)
     for (int d = 0; d < 3; ++d) {
@@ -409,29 +424,27 @@ void ifmm_tree::ensure_device() {
       dfp[(size_t)(2 * d) * N + i] = h;
       dfp[(size_t)(2 * d + 1) * N + i] = (float)(v - (double)h);
     }
-  CK(device_malloc((void**)&d_pts_df, sizeof(float) * 6 * N));
-  CK(cudaMemcpy(d_pts_df, dfp.data(), sizeof(float) * 6 * N, cudaMemcpyHostToDevice));
-  registry().add(d_pts, sizeof(double) * 3 * N);
-  registry().add(d_perm, sizeof(int32_t) * N);
-  registry().add(d_pts_df, sizeof(float) * 6 * N);
-  noalloc_prepare_device(device);
+  try {  // all copies or none: a later call takes what is there as complete
+    CK(device_malloc((void**)&d_pts, sizeof(double) * 3 * N));
+    pool_tree_count(1);
+    CK(cudaMemcpy(d_pts, soa.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice));
+    CK(device_malloc((void**)&d_perm, sizeof(int32_t) * N));
+    CK(cudaMemcpy(d_perm, perm.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
+    CK(device_malloc((void**)&d_pts_df, sizeof(float) * 6 * N));
+    CK(cudaMemcpy(d_pts_df, dfp.data(), sizeof(float) * 6 * N, cudaMemcpyHostToDevice));
+    registry().add(d_pts, sizeof(double) * 3 * N);
+    registry().add(d_perm, sizeof(int32_t) * N);
+    registry().add(d_pts_df, sizeof(float) * 6 * N);
+    noalloc_prepare_device(device);
+  } catch (...) {
+    release_device(*this);
+    throw;
+  }
 }
 
 ifmm_tree::~ifmm_tree() {
   fmm_free(fmm);
-  if (d_pts) {
-    registry().remove_range(d_pts, sizeof(double) * 3 * N);
-    cudaFree(d_pts);
-    pool_tree_count(-1);
-  }
-  if (d_perm) {
-    registry().remove_range(d_perm, sizeof(int32_t) * N);
-    cudaFree(d_perm);
-  }
-  if (d_pts_df) {
-    registry().remove_range(d_pts_df, sizeof(float) * 6 * N);
-    cudaFree(d_pts_df);
-  }
+  release_device(*this);
 }
 
 // Device buffers of one call, carved from one block of the pool: reserve() every
