@@ -2327,7 +2327,15 @@ void launch_m2m_table(cudaStream_t s, double* out, int p, int dof) {
   check_launch("k_m2m_table");
 }
 
-size_t matvec_part_doubles(int n, const ifmm_kernel& k) { return matvec64_part_doubles(n, kernel_dof(k)); }
+size_t matvec_part_doubles(int n, const ifmm_kernel& k) {
+  // IFMM_MATVEC64_FULL=1 (read once per process; tests): without partial sums, as where
+  // they would be too large
+  static const bool full = [] {
+    const char* e = getenv("IFMM_MATVEC64_FULL");
+    return e && e[0] == '1';
+  }();
+  return full ? 0 : matvec64_part_doubles(n, kernel_dof(k));
+}
 
 void launch_matvec(cudaStream_t s, const double* pts, int N, const double* x, double* y, const ifmm_kernel& k,
                    double* part) {

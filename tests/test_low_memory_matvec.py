@@ -48,3 +48,20 @@ assert product(t) == (0, 1)
 
 def test_full_sums_when_short_of_memory(tmp_path):
     fake_runtime.run(SCRIPT, tmp_path)
+
+
+FULL64 = r"""
+from paper_1905_10602_gb300.workloads import bumpy_sphere
+n = 3000
+t = ifmm.ifmm_build_tree(bumpy_sphere(n, 1), 3)
+ifmm.ifmm_color(t, 3)
+for k, x, name in ((ifmm.default_kernel(n), np.ones(n), "8k_matvecE"),
+                   (ifmm.helmholtz_kernel(n, 5.0), np.ones(n, complex), "10k_matvec_cE")):
+    fake.fake_clear()
+    ifmm.bem_matvec(t, x, kernel=k)
+    assert launches(name) == 1 and launches("k_matvec64_sym") == 0
+"""
+
+
+def test_switch_to_the_fp64_full_sums(tmp_path):
+    fake_runtime.run(FULL64, tmp_path, {"IFMM_MATVEC64_FULL": "1"})
