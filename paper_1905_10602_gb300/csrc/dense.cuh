@@ -1257,12 +1257,12 @@ __device__ __forceinline__ bool svd_needs(double al, double be, double g) {
 }
 // rotation that orthogonalises columns of squared norms al, be and product g:
 // t = tan, c = cos, s = sin; t^2 + 2 z t - 1 = 0 with z = (be - al) / (2 g).  Columns
-// of very different size have a z whose square leaves the FP32 range: there 1 / (2 z)
-// is the tangent to far below rounding (relative error 1 / (4 z^2)).
+// of very different size have a z whose square leaves the FP32 range: the root of
+// z^2 + 1 is at most |z| + 1, which is what counts there.
 __device__ __forceinline__ void svd_rotation(float al, float be, float g, float& t, float& c, float& s) {
   const float z = __fdividef(be - al, g + g);
-  const bool far = fabsf(z) > 1e9f;
-  t = __fdividef(far ? 0.5f : copysignf(1.f, z), far ? z : fabsf(z) + sqrt_fast(fmaf(z, z, 1.f)));
+  const float a = fabsf(z);
+  t = __fdividef(copysignf(1.f, z), a + fminf(sqrt_fast(fmaf(z, z, 1.f)), a + 1.f));
   const float x = fmaf(t, t, 1.f), y = rsqrtf(x);
   c = fmaf(0.5f * y, fmaf(-(x * y), y, 1.f), y);
   s = c * t;

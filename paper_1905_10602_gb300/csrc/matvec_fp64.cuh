@@ -18,7 +18,7 @@
 // k_matvec64_sum adds in tile order: no result depends on scheduling.
 //
 // One product through bem_matvec, device vectors: n = 10,007 Laplace 8.49 ms ->
-// 1.48 ms, n = 3,072 Helmholtz 10.7 ms -> 0.5 ms.  The full sums they
+// 1.32 ms, n = 3,072 Helmholtz 10.7 ms -> 0.5 ms.  The full sums they
 // replace had a thread per target and ceil(n / 256) CTAs.
 #pragma once
 
