@@ -45,22 +45,25 @@ sys.path.insert(0, ROOT)
 
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 METRIC = "IFMM factor+solve s at N=131k, eps=1e-6: mixed/learned vs plain FP64, same GB300"
-# FP32-pipe operations per pair interaction of the float-pair direct sum, counted
-# from its source (three pair differences, squares and their sum, the refined
-# reciprocal square root, the product with the charge and the accumulation)
-MATVEC_DF_OPS_PER_PAIR = 75
-# the symmetric kernel: one 1/r per unordered pair serves two entries; its
-# FP32 operations per evaluated pair (the 75 above plus the second product and
-# float-pair accumulation)
-MATVEC_SYM_OPS_PER_PAIR = 91
+# FP32 additions, multiplications and multiply-adds per evaluated pair of the
+# float-pair direct sums: of the plain kernel for one ordered pair, of the symmetric
+# one for an unordered pair, whose 1/r serves two entries (counted from the source;
+# ncu's counters read 89.0, and 89.6 with the symmetric kernel's diagonal tiles)
+MATVEC_DF_OPS_PER_PAIR = 89
+MATVEC_SYM_OPS_PER_PAIR = 88
+# FP64 operations per unordered pair of the FP64 direct sum (ncu: 13.2 with the
+# diagonal tiles)
+MATVEC64_OPS_PER_PAIR = 13
+# BF16 MMA passes of one FP64-grade product of the level-1 inverse (digit pairs)
+TOP_INVERSE_MMA_PASSES = 34
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) summed over the
 # kernels of each class in one factor + GMRES(30) of the bumpy sphere at
 # N = 32,768, depth 5, FP32 path: the --ncu-case command, captured with those
 # two metrics and gpu__time_duration.sum.  ncu flushes L2 before every launch,
 # so these are cold-cache bytes.  The classes listed have work linear in N at
 # fixed points per leaf; the default line scales them by N / 32,768.
-NCU_DRAM_BYTES_BUMPY32K = {"qr_fp32": 10.812e9, "svd_fp32": 0.411e9, "gemm_fp32": 18.600e9,
-                           "gauss_jordan": 0.117e9, "solve_graph": 1.636e9}
+NCU_DRAM_BYTES_BUMPY32K = {"qr_fp32": 12.585e9, "svd_fp32": 0.411e9, "gemm_fp32": 18.609e9,
+                           "gauss_jordan": 0.124e9, "solve_graph": 1.649e9}
 NCU_CAPTURE_N = 32768
 
 
@@ -299,15 +302,17 @@ def phase_rooflines(prof, stats, peaks, precision, n, its, steps_profiled=1, mat
     add(sk, "a6 recompression Jacobi SVD", stats.get("flops_svd", 0.0), "TFLOP/s", "alu",
         peaks["fp64" if precision == "fp64" else "fp32"], "FP64 FMA peak" if precision == "fp64" else "FP32 FMA peak")
     add("gauss_jordan", "a4 pivot inverses (FP64)", stats.get("flops_inv", 0.0), "TFLOP/s", "alu", peaks["fp64"], "FP64 FMA peak")
-    add("gauss_jordan_big", "a9 level-1 inverse (FP64)", stats.get("flops_lu", 0.0), "TFLOP/s", "alu", peaks["fp64"],
-        "FP64 FMA peak")
+    add("gauss_jordan_big", "a9 level-1 inverse (FP64)", stats.get("flops_lu", 0.0), "TFLOP/s", "tensor",
+        peaks["bf16_mma"] / TOP_INVERSE_MMA_PASSES,
+        f"BF16 warp MMA peak / {TOP_INVERSE_MMA_PASSES} (passes over 8-bit digits per product)")
     apps = its + 1  # preconditioner applications per GMRES solve (one per iteration, one for x)
     add("solve_graph", "a10 IFMM solve (preconditioner)", stats.get("solve_matrix_bytes", 0.0) * apps, "GB/s", "hbm",
         peaks["hbm_gbs"], "HBM copy bandwidth")
     matvec = matvec or ("fp64" if precision == "fp64" else "df")
     if matvec == "fp64":
-        add("matvec", "a11 direct-sum matvec (FP64)", 20.0 * n * n * (its + 1), "TFLOP/s", "alu", peaks["fp64"],
-            "FP64 FMA peak, ~20 flops per pair")
+        add("matvec", "a11 direct-sum matvec (FP64, symmetric)", n * (n - 1) / 2.0 * (its + 1), "Gpairs/s", "alu",
+            peaks["fp64"] * 1e3 / 2.0 / MATVEC64_OPS_PER_PAIR,
+            f"measured FP64 FMA issue rate / {MATVEC64_OPS_PER_PAIR} FP64 operations per unordered pair")
     elif matvec == "df":
         n_, ms = prof.get("matvec", (0, 0.0))
         if n_ and ms > 0:
