@@ -7,7 +7,7 @@
 // start values of 1/r come from the FP32 reciprocal square root of the leading
 // bits, moved between the formats by integer operations, and sine and cosine
 // from a 64-entry table of one turn plus short Taylor sums.  13 FP64 operations
-// per unordered pair (Laplace), 44 (Helmholtz).
+// per unordered pair (Laplace), 43 (Helmholtz).
 //
 // The points are cut into tiles of TB; a CTA takes a pair of tiles I <= J, each
 // warp holding 32 targets of tile I and walking the sources of tile J in chunks
