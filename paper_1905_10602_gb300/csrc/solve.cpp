@@ -451,9 +451,25 @@ ifmm_tree::~ifmm_tree() {
 // piece first, then get() them.
 struct Vecs {
   char* base = nullptr;
-  size_t total = 0, off = 0;
+  size_t total = 0, off = 0, extra = 0;
   static size_t up(size_t n) { return (sizeof(double) * std::max<size_t>(n, 1) + 255) & ~(size_t)255; }
   void reserve(size_t n) { total += up(n); }
+  // Takes the block, after every reserve(), with n more doubles that a faster kernel
+  // wants and the call can do without: null when n is 0 or the device has no room for
+  // them (the block is then taken without them).
+  double* take_with(size_t n) {
+    if (!n) return nullptr;
+    try {
+      base = (char*)pool_alloc(total + up(n));
+    } catch (const Error& e) {
+      if (e.code != IFMM_ENOMEM) throw;
+      return nullptr;
+    }
+    double* x = (double*)(base + total);
+    registry().add(x, sizeof(double) * n);
+    extra = up(n);
+    return x;
+  }
   double* get(size_t n) {
     if (!base) base = (char*)pool_alloc(std::max<size_t>(total, 256));
     IFMM_REQUIRE(off + up(n) <= total, IFMM_EINVAL, "internal: workspace larger than reserved");
@@ -468,7 +484,7 @@ struct Vecs {
   ~Vecs() {
     if (!base) return;
     pool_quiesce();
-    registry().remove_range(base, total);
+    registry().remove_range(base, total + extra);
     pool_free(base);
   }
 };
@@ -592,8 +608,9 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
     const bool df_mv = k->arith == IFMM_ARITH_DF, fmm_mv = k->arith == IFMM_ARITH_FMM;
     // partial sums of the symmetric kernels
     const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
-    Vecs V, W;
+    Vecs V;
     for (int i = 0; i < (df_mv ? 4 : 3); ++i) V.reserve(N);
+    double* part = V.take_with(np);
     double* a = V.get(N);
     double* b = V.get(N);
     double* c = V.get(N);
@@ -610,14 +627,13 @@ ifmm_status bem_matvec(const ifmm_tree* t, const ifmm_kernel* k, const double* x
       float* q = (float*)V.get(N);
       launch_split_df(s, a, q, q + N, (int)N);
       ifmm_tree* tm = const_cast<ifmm_tree*>(t);
-      float2* part = np ? (float2*)get_or_null(W, np) : nullptr;
       const bool short_of_memory = np && !part;
       const int tile = tm->matvec_block && !short_of_memory
                            ? tm->matvec_block
-                           : matvec_tile(tm, s, q, a, b, N, k, part, short_of_memory);
-      launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, part);
+                           : matvec_tile(tm, s, q, a, b, N, k, (float2*)part, short_of_memory);
+      launch_matvec_df(s, t->d_pts_df, q, q + N, a, b, (int)N, k->scale, k->diag, tile, (float2*)part);
     } else {
-      launch_matvec(s, t->d_pts, (int)NP, a, b, *k, np ? get_or_null(W, np) : nullptr);
+      launch_matvec(s, t->d_pts, (int)NP, a, b, *k, part);
     }
     if (dev) {
       launch_scatter_perm(s, b, t->d_perm, y, (int)NP, dof);
@@ -658,12 +674,13 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     // another kernel, or FP64)
     const size_t np = df_mv ? sym_part_doubles(*t) : (fmm_mv ? 0 : matvec_part_doubles((int)NP, *k));
     const size_t nkp = (size_t)kry_parts(N) * 2 * m;
-    Vecs Vm, W;
+    Vecs Vm;
     for (int i = 0; i < 6; ++i) Vm.reserve(N);
     Vm.reserve((size_t)N * (m + 1));
     Vm.reserve(2 * (size_t)m + 2);
     Vm.reserve(nkp);
     if (df_mv) Vm.reserve(N);
+    double* part = Vm.take_with(np);
     double* bt = Vm.get(N);   // b in tree order
     double* xt = Vm.get(N);   // x in tree order
     double* rt = Vm.get(N);
@@ -674,7 +691,6 @@ ifmm_status bem_gmres(const ifmm_tree* t, const ifmm_kernel* k, const ifmm_fact*
     double* kp = Vm.get(nkp);
     double* tmp = Vm.get(N);
     float* qdf = df_mv ? (float*)Vm.get(N) : nullptr;
-    double* part = np ? get_or_null(W, np) : nullptr;
     const double* src = b;
     if (!dev) {
       CK(cudaMemcpyAsync(tmp, b, sizeof(double) * N, cudaMemcpyHostToDevice, s));
